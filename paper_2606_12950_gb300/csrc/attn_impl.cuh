@@ -8,8 +8,9 @@
 // evaluated with an online softmax in base 2 and fp32 accumulation.
 //
 // Work decomposition (all decided on the device from the lengths):
-//   unit  = one 16-token tile of one (sequence, KV head) run; a run of n
-//           tokens has ceil(n/16) units; units are ordered (s, g, tile).
+//   unit  = one tile of one (sequence, KV head) run: 16 tokens at d = 128,
+//           32 at d = 64 (kUnit), 8 KB of K and V either way; a run of n
+//           tokens has ceil(n/kUnit) units; units are ordered (s, g, tile).
 //   part  = one of NP = P * 8 equal contiguous unit ranges [i*W/NP,
 //           (i+1)*W/NP), one per warp of the P resident CTAs: every warp
 //           streams the same number of bytes (+-1 tile) whatever the length
@@ -70,8 +71,22 @@ constexpr int kWarps = 8;
 constexpr int kThreads = kWarps * 32;
 constexpr int kPlainWarps = 6;
 constexpr int kStages = 1;  // units in flight per warp (each a K and a V tile)
-constexpr int kTile = 16;                         // tokens per unit
-constexpr int kMinUnitsPerPart = 4;
+constexpr int kTile = 16;                         // tokens per TMA box: the least block size
+// Tokens per unit.  A warp's work on a unit is one dependent chain (wait for
+// K, q.K, softmax, wait for V, P.V, the next requests) of much the same
+// length whatever d is.  At d = 64 a 16-token unit is only 4 KB, and that
+// chain, not HBM, set the pace: 128 sequences of lognormal length (209k
+// tokens, 32 q / 8 KV heads, 429 MB) took 83.2 us a step with 16-token units
+// (78.9 with two units in flight a warp, 79.7 with eight warps a CTA) and
+// 75.1 with 32-token ones, which bring d = 64 to the bytes per chain of
+// d = 128 (5.7 against 5.2 TB/s).
+template <int D>
+constexpr int kUnit = D == 64 ? 32 : 16;
+template <int D>
+constexpr int kSub = kUnit<D> / kTile;            // boxes' rows per unit
+// a part's least tokens (4 units at d = 128, 2 at d = 64): with 128 at d = 64
+// a step of four short sequences took 18.5 us instead of 15.5
+constexpr int kMinPartTokens = 64;
 constexpr uint32_t kHalfBytes = kTile * 128;      // one 64-column box: 16 rows x 128 B
 constexpr uint64_t kWaitLimitNs = 2000000000ull;  // bounded mbarrier waits: 2 s
 
@@ -110,7 +125,7 @@ struct AttnArgs {
     int32_t S;
     int32_t Hkv;
     int32_t bs;
-    int32_t rows_cap;        // units whose pool rows are resolved up front
+    int32_t rows_cap;        // boxes whose pool rows are resolved up front
     int32_t P;               // CTAs
     int32_t nwarps;          // warps per CTA (<= kWarps), one part each
     float qk_scale;          // scale * log2(e)
@@ -204,7 +219,7 @@ struct FmaCompute {
     static constexpr int EPL = D / LPT;                      // elements per lane
     static constexpr int NCH = EPL / 8;                      // 16-byte chunks per lane
     static constexpr int NGRP = 32 / LPT;                    // tokens in flight per warp
-    static constexpr int TPG = kTile / NGRP;                 // tokens per group per tile
+    static constexpr int TPG = kUnit<D> / NGRP;              // tokens per group per unit
     static_assert(EPL % 8 == 0, "lane slice must be whole 16-byte chunks");
 
     float2 q[G][EPL / 2];
@@ -382,10 +397,11 @@ struct MmaCompute {
     static_assert(G <= 8, "query-head group must fit the n=8 MMA tile");
     static constexpr int kMinBlocks = 2;
     static constexpr int KS = D / 16;
+    static constexpr int NM = kSub<D>;  // 16-token MMA tiles per unit
     uint32_t qf[KS][2];  // B operand of q.K: Q^T fragments (bf16x2)
     float acc[KS][4];    // O^T accumulators, 16 d-rows per block
     float m[2], l[2];    // heads 2*tig, 2*tig+1
-    uint32_t pb0, pb1;   // B operand of P.V (P^T fragments)
+    uint32_t pb[NM][2];  // B operand of P.V (P^T fragments)
     float qk_scale;
     int gid, tig, lane_, nv;
 
@@ -417,20 +433,32 @@ struct MmaCompute {
         nv = nvalid;
         const uint32_t kbase = smem_u32(Ks);
         const int mat = lane_ >> 3, r8 = lane_ & 7;
-        float s[4] = {0.f, 0.f, 0.f, 0.f};
+        // rows past the valid tokens of a loaded box may hold anything; a box
+        // that was not loaded (16 mt >= nvalid) holds an earlier
+        // unit's rows: both are masked
+        float x[NM][4];
 #pragma unroll
-        for (int kk = 0; kk < KS; ++kk) {
-            uint32_t a0, a1, a2, a3;
-            ldmatrix_x4(kbase + swz(r8 + (mat & 1) * 8, kk * 2 + (mat >> 1)), a0, a1, a2, a3);
-            mma_bf16_16816(s, a0, a1, a2, a3, qf[kk][0], qf[kk][1]);
+        for (int mt = 0; mt < NM; ++mt) {
+            float s[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+            for (int kk = 0; kk < KS; ++kk) {
+                uint32_t a0, a1, a2, a3;
+                ldmatrix_x4(kbase + swz(mt * 16 + r8 + (mat & 1) * 8, kk * 2 + (mat >> 1)), a0, a1, a2, a3);
+                mma_bf16_16816(s, a0, a1, a2, a3, qf[kk][0], qf[kk][1]);
+            }
+            // s[0], s[1]: token gid, heads 2tig, 2tig+1; s[2], s[3]: token gid+8
+            const bool ok0 = mt * 16 + gid < nvalid, ok1 = mt * 16 + gid + 8 < nvalid;
+            x[mt][0] = ok0 ? s[0] * qk_scale : -INFINITY;
+            x[mt][1] = ok0 ? s[1] * qk_scale : -INFINITY;
+            x[mt][2] = ok1 ? s[2] * qk_scale : -INFINITY;
+            x[mt][3] = ok1 ? s[3] * qk_scale : -INFINITY;
         }
-        // s[0], s[1]: token gid, heads 2tig, 2tig+1; s[2], s[3]: token gid+8
-        const bool ok0 = gid < nvalid, ok1 = gid + 8 < nvalid;
-        const float x0 = ok0 ? s[0] * qk_scale : -INFINITY;
-        const float x1 = ok0 ? s[1] * qk_scale : -INFINITY;
-        const float x2 = ok1 ? s[2] * qk_scale : -INFINITY;
-        const float x3 = ok1 ? s[3] * qk_scale : -INFINITY;
-        float t0 = fmaxf(x0, x2), t1 = fmaxf(x1, x3);
+        float t0 = fmaxf(x[0][0], x[0][2]), t1 = fmaxf(x[0][1], x[0][3]);
+#pragma unroll
+        for (int mt = 1; mt < NM; ++mt) {
+            t0 = fmaxf(t0, fmaxf(x[mt][0], x[mt][2]));
+            t1 = fmaxf(t1, fmaxf(x[mt][1], x[mt][3]));
+        }
 #pragma unroll
         for (int off = 4; off < 32; off <<= 1) {
             t0 = fmaxf(t0, __shfl_xor_sync(0xffffffffu, t0, off));
@@ -457,22 +485,25 @@ struct MmaCompute {
             }
             m[1] = t1;
         }
-        const float p0 = fast_exp2(x0 - m[0]), p1 = fast_exp2(x1 - m[1]);
-        const float p2 = fast_exp2(x2 - m[0]), p3 = fast_exp2(x3 - m[1]);
-        l[0] += p0 + p2;
-        l[1] += p1 + p3;
-        __nv_bfloat162 lo = __floats2bfloat162_rn(p0, p1);
-        __nv_bfloat162 hi = __floats2bfloat162_rn(p2, p3);
-        pb0 = movmatrix_trans(*reinterpret_cast<uint32_t *>(&lo));
-        pb1 = movmatrix_trans(*reinterpret_cast<uint32_t *>(&hi));
+#pragma unroll
+        for (int mt = 0; mt < NM; ++mt) {
+            const float p0 = fast_exp2(x[mt][0] - m[0]), p1 = fast_exp2(x[mt][1] - m[1]);
+            const float p2 = fast_exp2(x[mt][2] - m[0]), p3 = fast_exp2(x[mt][3] - m[1]);
+            l[0] += p0 + p2;
+            l[1] += p1 + p3;
+            __nv_bfloat162 lo = __floats2bfloat162_rn(p0, p1);
+            __nv_bfloat162 hi = __floats2bfloat162_rn(p2, p3);
+            pb[mt][0] = movmatrix_trans(*reinterpret_cast<uint32_t *>(&lo));
+            pb[mt][1] = movmatrix_trans(*reinterpret_cast<uint32_t *>(&hi));
+        }
     }
 
     __device__ __forceinline__ void pv(uint8_t *Vs)
     {
         // rows past the context may hold anything (even NaN bit patterns);
         // P is zero there, but 0 * NaN is NaN inside the MMA, so clear them
-        if (nv < kTile) {
-            const int nchunk = (kTile - nv) * (D / 8);
+        if (nv < kUnit<D>) {
+            const int nchunk = (kUnit<D> - nv) * (D / 8);
             for (int idx = lane_; idx < nchunk; idx += 32) {
                 const int r = nv + idx / (D / 8);
                 const int c = idx % (D / 8);
@@ -484,9 +515,12 @@ struct MmaCompute {
         const int mat = lane_ >> 3, r8 = lane_ & 7;
 #pragma unroll
         for (int mb = 0; mb < KS; ++mb) {
-            uint32_t a0, a1, a2, a3;
-            ldmatrix_x4_trans(vbase + swz(r8 + (mat >> 1) * 8, mb * 2 + (mat & 1)), a0, a1, a2, a3);
-            mma_bf16_16816(acc[mb], a0, a1, a2, a3, pb0, pb1);
+#pragma unroll
+            for (int mt = 0; mt < NM; ++mt) {
+                uint32_t a0, a1, a2, a3;
+                ldmatrix_x4_trans(vbase + swz(mt * 16 + r8 + (mat >> 1) * 8, mb * 2 + (mat & 1)), a0, a1, a2, a3);
+                mma_bf16_16816(acc[mb], a0, a1, a2, a3, pb[mt][0], pb[mt][1]);
+            }
         }
     }
 
@@ -624,17 +658,21 @@ __device__ __forceinline__ int32_t table_entry(const AttnArgs &a, int64_t idx)
     return ld_prior(a.table + idx, a.chain >= 2);
 }
 
-// Pool row of unit u's K tile (TMA y coordinate; V is Hkv*bs rows further),
-// or -1 if the block table names a block outside the pool.
-__device__ __forceinline__ int32_t unit_row(const AttnArgs &a, const int32_t *T, int32_t u)
+// Pool row of box j of unit u's K tile (TMA y coordinate; V is Hkv*bs rows
+// further), kRowBad if the block table names a block outside the pool, or
+// kRowNone if the context ends before the box (the table may have no entry).
+constexpr int32_t kRowBad = -1, kRowNone = -2;
+template <int D>
+__device__ __forceinline__ int32_t unit_row(const AttnArgs &a, const int32_t *T, int32_t u, int j)
 {
     const int s = find_seq(T, a.S, u);
     const int32_t nt = (T[s + 1] - T[s]) / a.Hkv;
     const int32_t within = u - T[s];
     const int32_t g = within / nt;
-    const int32_t tok0 = seq_skip(T, a.S, s) + (within - g * nt) * kTile;
+    const int32_t tok0 = seq_skip(T, a.S, s) + (within - g * nt) * kUnit<D> + j * kTile;
+    if (j > 0 && tok0 >= seq_len(T, a.S, s)) return kRowNone;
     const int32_t phys = table_entry(a, (int64_t)s * a.max_blocks + tok0 / a.bs);
-    if (phys < 0 || (int64_t)phys + a.pages_per_block > a.pool_pages) return -1;
+    if (phys < 0 || (int64_t)phys + a.pages_per_block > a.pool_pages) return kRowBad;
     return (int32_t)((int64_t)phys * a.rows_per_page + (tok0 % a.bs) + (int64_t)g * a.bs);
 }
 
@@ -656,18 +694,29 @@ __device__ __forceinline__ void issue_half(const CUtensorMap *tmap, const AttnAr
                                            const int32_t *rows, int32_t cu0, int32_t u, int which, uint32_t dst,
                                            uint32_t bar, uint64_t policy)
 {
-    constexpr int HALVES = D / 64;
-    const int32_t k = u - cu0;
-    int32_t y = k < a.rows_cap ? rows[k] : unit_row(a, T, u);
-    if (y < 0) {
+    constexpr int HALVES = D / 64, SUB = kSub<D>;
+    const int32_t k = (u - cu0) * SUB;
+    int32_t y[SUB];
+    uint32_t boxes = 0;
+    bool bad = false;
+#pragma unroll
+    for (int j = 0; j < SUB; ++j) {
+        y[j] = k + j < a.rows_cap ? rows[k + j] : unit_row<D>(a, T, u, j);
+        bad |= y[j] == kRowBad;
+        boxes += y[j] >= 0 ? 1u : 0u;
+    }
+    if (bad) {
         report(a.err, KV_ERR_DEVICE_BOUNDS);
         mbar_arrive(bar);  // complete the phase without data
         return;
     }
-    y += which * a.Hkv * a.bs;
-    mbar_arrive_expect_tx(bar, HALVES * kHalfBytes);
+    mbar_arrive_expect_tx(bar, boxes * HALVES * kHalfBytes);
 #pragma unroll
-    for (int h = 0; h < HALVES; ++h) tma_load_2d(dst + h * kHalfBytes, tmap, h * 64, y, bar, policy);
+    for (int j = 0; j < SUB; ++j)
+        if (SUB == 1 || y[j] >= 0)
+#pragma unroll
+            for (int h = 0; h < HALVES; ++h)  // box (j, h): with SUB > 1, HALVES is 1
+                tma_load_2d(dst + (j + h) * kHalfBytes, tmap, h * 64, y[j] + which * a.Hkv * a.bs, bar, policy);
 }
 
 template <int D, int G, class Comp>
@@ -675,7 +724,9 @@ __global__ void __launch_bounds__(kThreads, Comp::kMinBlocks)
 paged_attn_kernel(const __grid_constant__ CUtensorMap tmap, const __grid_constant__ AttnArgs a)
 {
     constexpr int HALVES = D / 64;
-    constexpr uint32_t TILE_BYTES = HALVES * kHalfBytes;
+    constexpr int UNIT = kUnit<D>, SUB = kSub<D>;
+    static_assert(HALVES == 1 || SUB == 1, "a unit's boxes follow each other in shared memory");
+    constexpr uint32_t TILE_BYTES = HALVES * SUB * kHalfBytes;
     constexpr uint32_t STAGE_BYTES = 2 * TILE_BYTES;
     constexpr uint32_t MF = merge_floats<D, G>();
     extern __shared__ uint8_t smem_raw[];
@@ -765,7 +816,7 @@ paged_attn_kernel(const __grid_constant__ CUtensorMap tmap, const __grid_constan
             NL[s] = n | (raw != n ? (int32_t)0x80000000 : 0);
             SK[s] = k;
             const int32_t ne = n - k;
-            local += ((ne + kTile - 1) / kTile) * Hkv;
+            local += ((ne + UNIT - 1) / UNIT) * Hkv;
         }
         int32_t incl = local;
 #pragma unroll
@@ -780,7 +831,7 @@ paged_attn_kernel(const __grid_constant__ CUtensorMap tmap, const __grid_constan
         int32_t run = base + incl - local;
         for (int s = lo; s < hi; ++s) {  // this thread's own NL / SK entries
             T[s] = run;
-            run += ((seq_len(T, S, s) - seq_skip(T, S, s) + kTile - 1) / kTile) * Hkv;
+            run += ((seq_len(T, S, s) - seq_skip(T, S, s) + UNIT - 1) / UNIT) * Hkv;
         }
         if (tid == 0) {
             int32_t tot = 0;
@@ -811,10 +862,11 @@ paged_attn_kernel(const __grid_constant__ CUtensorMap tmap, const __grid_constan
     // [i*W/NP, (i+1)*W/NP) and belongs to warp i % NW of CTA i / NW.
     // With NP <= W every part is non-empty, so a run's contributors are
     // exactly the parts part_of(first unit) .. part_of(last unit).  A part
-    // gets at least kMinUnitsPerPart units when the batch is small (fewer
+    // gets at least MIN_UNITS units when the batch is small (fewer
     // partials to write and merge; enough warps still stream to fill HBM).
     const int64_t W = T[S];
-    const int64_t np_min = W > 0 ? (W / kMinUnitsPerPart > 0 ? W / kMinUnitsPerPart : 1) : 0;
+    constexpr int MIN_UNITS = kMinPartTokens / UNIT;
+    const int64_t np_min = W > 0 ? (W / MIN_UNITS > 0 ? W / MIN_UNITS : 1) : 0;
     const int64_t NP = np_min < (int64_t)a.P * NW ? np_min : (int64_t)a.P * NW;
     const int64_t first_part = (int64_t)blockIdx.x * NW;
     if (first_part >= NP) {
@@ -828,8 +880,8 @@ paged_attn_kernel(const __grid_constant__ CUtensorMap tmap, const __grid_constan
     // ---- prologue 2: resolve the block table for this CTA's units while the
     // memory system is idle (later lookups would queue behind the TMA stream)
     {
-        const int32_t nr = min(cu1 - cu0, a.rows_cap);
-        for (int32_t k = tid; k < nr; k += NT) rows[k] = unit_row(a, T, cu0 + k);
+        const int32_t nr = min((cu1 - cu0) * SUB, a.rows_cap);
+        for (int32_t k = tid; k < nr; k += NT) rows[k] = unit_row<D>(a, T, cu0 + k / SUB, k % SUB);
         __syncthreads();
     }
 
@@ -899,10 +951,10 @@ paged_attn_kernel(const __grid_constant__ CUtensorMap tmap, const __grid_constan
             uint8_t *Ks = k_of(st);
             uint8_t *Vs = Ks + TILE_BYTES;
             const uint32_t bk = bk_of(st), bv = bv_of(st);
-            const int nvalid = min(kTile, pc.n - pc.skip - (uu - pc.run_begin) * kTile);
+            const int nvalid = min(UNIT, pc.n - pc.skip - (uu - pc.run_begin) * UNIT);
             const bool more = uu + kStages < u1;  // the unit this stage takes next
             const bool app = app_run && uu == pc.run_end - 1;
-            const int arow = (pc.n - 1) % kTile;
+            const int arow = (pc.n - 1 - pc.skip) % UNIT;
             wait_phase(bk, par, a.err, dead);
             if (app) {
                 cp_async_wait_all();  // the new K/V rows
@@ -928,11 +980,12 @@ paged_attn_kernel(const __grid_constant__ CUtensorMap tmap, const __grid_constan
             if (app) {
                 // store the new row into the pool: this warp's own TMA reads of
                 // the tile have completed, and no other unit covers that row
-                const int32_t k = uu - cu0;
-                const int32_t y = k < a.rows_cap ? rows[k] : unit_row(a, T, uu);
+                const int j = arow / kTile;  // the box that holds the row
+                const int32_t k = (uu - cu0) * SUB + j;
+                const int32_t y = k < a.rows_cap ? rows[k] : unit_row<D>(a, T, uu, j);
                 if (y >= 0 && lane < AB / 16) {
                     const int which = lane / (D / 8), c = lane % (D / 8);
-                    const int64_t row = (int64_t)y + arow + (int64_t)which * Hkv * a.bs;
+                    const int64_t row = (int64_t)y + arow % kTile + (int64_t)which * Hkv * a.bs;
                     *reinterpret_cast<uint4 *>(a.pool + row * D + c * 8) =
                         *reinterpret_cast<const uint4 *>(ab + lane * 16);
                 }
@@ -1154,7 +1207,7 @@ constexpr int kRowsCap = 2048;
 template <int D, int G>
 inline size_t attn_smem_bytes(int S, int rows_cap, int nwarps)
 {
-    const size_t stage = 2ull * (D / 64) * kHalfBytes;
+    const size_t stage = 2ull * (D / 64) * kSub<D> * kHalfBytes;
     const size_t bufs = (size_t)G * D * 2 + 2 * D * 2;  // per warp: q rows, new K/V rows
     return 1024 + (size_t)nwarps * (kStages * stage + bufs) + (2 * nwarps * kStages) * 8 + 64 + (size_t)(3 * S + 1) * 4 +
            (size_t)rows_cap * 4;

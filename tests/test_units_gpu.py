@@ -1,0 +1,70 @@
+"""GPU parity at the edges of the decode kernel's work split: contexts that
+end just before, at and after the edges of a 16-token box and of a unit (16
+tokens at d = 128, 32 at d = 64), against the fp64 oracle.
+
+Bars as in test_parity_gpu.py (max |err| <= 1.5e-2, mean |err| <= 2e-3, the
+pool bit-exact): bf16 outputs of fp32 sums over N(0, 1) values.
+"""
+import numpy as np
+import pytest
+
+import oracle
+from paper_2606_12950_gb300 import workloads as W
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+MAX_ABS = 1.5e-2
+MEAN_ABS = 2e-3
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _cuda():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+
+
+def _check(got, ref, what):
+    err = np.abs(got - ref)
+    assert np.isfinite(got).all(), what
+    assert err.max() <= MAX_ABS and err.mean() <= MEAN_ABS, (what, err.max(), err.mean())
+
+
+def _nan_past_contexts(b):
+    """NaN bit patterns in every row of a sequence's blocks past its context,
+    and in every block that no sequence holds."""
+    view = b.pool.reshape(b.n_pages, 2, b.Hkv, b.bs, b.d)
+    held = np.zeros(b.n_pages, bool)
+    for s in range(b.S):
+        n = int(b.ctx_lens[s])
+        blocks = b.table[s, : -(-n // b.bs)]
+        held[blocks] = True
+        if n % b.bs:
+            view[blocks[-1], :, :, n % b.bs:, :] = 0xFFFF
+    view[~held] = 0xFFFF
+
+
+@pytest.mark.parametrize("fused", [False, True], ids=["separate", "fused"])
+@pytest.mark.parametrize("variant", [1, 2])
+@pytest.mark.parametrize("bs", [16, 32, 64])
+@pytest.mark.parametrize("d", [64, 128])
+def test_context_lengths_at_box_and_unit_edges(d, bs, variant, fused):
+    from paper_2606_12950_gb300.runner import DeviceBatch, DevicePool
+
+    pre = [0, 14, 15, 16, 30, 31, 32, 46, 47, 48, 62, 63, 64, 95, 127, 500, 1023]
+    b = W.make_batch(7000 + d + bs, pre, Hq=8, Hkv=2, d=d, bs=bs, extra_blocks=5)
+    _nan_past_contexts(b)
+    pool = DevicePool(b.n_pages, b.page_elems * 2, b.bs, [(b.Hkv, b.d)])
+    pool.upload(b.pool)
+    pool.set_variant(variant)
+    db = DeviceBatch(pool, 0, b)
+    if fused:
+        db.append_attend()
+    else:
+        db.append()
+        db.attend()
+    torch.cuda.synchronize()
+    ref_pool = oracle.batch_append(b)
+    assert np.array_equal(pool.download(), ref_pool)
+    _check(db.out_f64(), oracle.batch_attention(b, pool=ref_pool), (d, bs, variant, fused))
+    assert pool.error() == 0
