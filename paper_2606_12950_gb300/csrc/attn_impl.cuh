@@ -687,6 +687,30 @@ __device__ __forceinline__ int32_t cta_of(int64_t u, int64_t W, int64_t P)
 template <int D, int G>
 __host__ __device__ constexpr uint32_t merge_floats() { return (G * D + 2 * G + 3) / 4 * 4; }
 
+// one more record (m, l, o) of a run into its merged state (M, L, O), for one
+// float4 column: base-2 online softmax.  A record without tokens (m = -inf)
+// leaves the state as it is.
+__device__ __forceinline__ void merge_record(float &M, float &L, float4 &O, float m, float l, const float4 &o)
+{
+    if (m == -INFINITY) return;
+    const float Mn = fmaxf(M, m);
+    const float sa = fast_exp2(M - Mn), sb = fast_exp2(m - Mn);
+    L = L * sa + l * sb;
+    O.x = O.x * sa + o.x * sb;
+    O.y = O.y * sa + o.y * sb;
+    O.z = O.z * sa + o.z * sb;
+    O.w = O.w * sa + o.w * sb;
+    M = Mn;
+}
+
+// a merged column's four outputs, bf16(O / L)
+__device__ __forceinline__ void store_column(uint16_t *dst, const float4 &O, float L)
+{
+    __nv_bfloat162 lo = __floats2bfloat162_rn(O.x / L, O.y / L);
+    __nv_bfloat162 hi = __floats2bfloat162_rn(O.z / L, O.w / L);
+    *reinterpret_cast<uint2 *>(dst) = make_uint2(*reinterpret_cast<uint32_t *>(&lo), *reinterpret_cast<uint32_t *>(&hi));
+}
+
 // Load K (which = 0) or V (which = 1) of unit u into this warp's stage;
 // completes on `bar`.  Lane 0 only.
 template <int D>
@@ -1017,11 +1041,13 @@ paged_attn_kernel(const __grid_constant__ CUtensorMap tmap, const __grid_constan
 // Split-K combine: for each (sequence, KV head) run cut by part boundaries
 // (or with a shared prefix), merge its records (m_k, l_k, o_k) in order:
 //     M = max_k m_k,  out = sum_k 2^(m_k - M) o_k / sum_k 2^(m_k - M) l_k
-// (base-2 online-softmax state).  One CTA per run, covering all G*D output
-// columns: NG thread groups of G*D/(4*CPT) threads (CPT float4 columns
-// each) take records k = grp, grp + NG, ..., then merge their states in
-// group order, so the result depends only on the run's shape.  Runs finished
-// inside the attention kernel return at once.
+// (base-2 online-softmax state).  CS CTAs per run, each covering a CS-th of its
+// G*D output columns: NG thread groups of G*D/(4*CPT*CS) threads (CPT float4
+// columns each) take records k = grp, grp + NG, ..., then merge their states
+// by halves in a fixed order, so the result depends only on the run's shape.
+// (Merged one after another by the first group, 29 groups made a step of four
+// short sequences 3 µs longer: 15.4 µs against 12.4.)  Runs finished inside
+// the attention kernel return at once.
 struct CombineArgs {
     uint16_t *out;
     const int2 *ws_run;    // per run: (first part, parts), parts = 0 when not split
@@ -1036,24 +1062,33 @@ struct CombineArgs {
 constexpr int kCombineMaxThreads = 1024;
 constexpr int kCombineBatch = 8;  // records each thread loads per round trip
 
-// Thread groups per combine CTA (a run's records are spread over the
-// groups, kCombineBatch loads in flight per thread): enough groups for
-// about 8 records per thread, up to 1024 threads, and at least 128 threads
-// (one group when a run's output has 128 float4 columns or more).  Small
-// CTAs leave room on the SMs for the next step's decode CTAs, which start
-// as the combine's CTAs finish: on the Llama-3-8B-shaped layer (64
-// sequences, 32 q / 8 KV heads) 128-thread CTAs took 54.5-54.9 µs per step
-// against 55.1-55.4 with 256 (six same-box pairs), at a cost of about 1 µs
-// in 296 for three co-located models, whose heavy-tailed runs take more
-// round trips with one group.
-template <int D, int G>
-inline int combine_groups(double records_per_run, bool shared_prefix)
+// CTAs per run (CS) and thread groups per combine CTA.
+//
+// Where each run has a CTA (CS = 1; kCombineBatch loads in flight per
+// thread): enough groups for about 8 records per thread, up to 1024 threads,
+// and at least 128 threads (one group when a run's output has 128 float4
+// columns or more).  Small CTAs leave room on the SMs for the next step's
+// decode CTAs, which start as the combine's CTAs finish: on the
+// Llama-3-8B-shaped layer (64 sequences, 32 q / 8 KV heads) 128-thread CTAs
+// took 54.5-54.9 µs per step against 55.1-55.4 with 256 (six same-box
+// pairs), at a cost of about 1 µs in 296 for three co-located models, whose
+// heavy-tailed runs take more round trips with one group.
+//
+// Few runs leave most SMs idle while one SM fetches a run's records (one
+// sequence of 8193 tokens: 8 runs of 128 records, 2 MB through 8 SMs, 8.9 µs
+// of a 22 µs step).  Up to kSlicedCtas CTAs an SM, a run's columns are spread
+// over 8 or 4 CTAs, each with groups for about 8 records a thread, at most
+// 16.  That step: 20.7 µs with CS = 1 and 15.8 with CS = 8 (both with the
+// groups merged by halves, below).  The line, on 64 runs of 6 records (8
+// sequences, 40 q / 8 KV heads, CTA-level parts): CS = 8 19.9 µs, CS = 1 20.2.
+constexpr int kSlicedCtas = 4;
+template <int D, int G, int CS>
+inline int combine_groups(double records_per_run)
 {
-    constexpr int NC = G * D / 4;
-    (void)shared_prefix;
-    const int floor_threads = 128;
+    constexpr int NC = G * D / 4 / CS;
+    constexpr int floor_threads = CS == 1 ? 128 : 64;
     const int base = NC >= floor_threads ? 1 : floor_threads / NC;
-    const int most = kCombineMaxThreads / NC;
+    const int most = CS == 1 ? kCombineMaxThreads / NC : (16 > base ? 16 : base);
     int want = (int)(records_per_run / 8.0 + 0.999);
     return want < base ? base : (want > most ? most : want);
 }
@@ -1065,9 +1100,9 @@ inline int combine_groups(double records_per_run, bool shared_prefix)
 // columns a thread (64 threads a run, registers held to 64, no shared
 // memory) sixteen fit and one wave covers 2432 runs.  Each column merges the
 // same records in the same order either way, so the bits do not change.
-template <int D, int G, int CPT>
+template <int D, int G, int CPT, int CS = 1>
 struct CombineShape {
-    static constexpr int NC = G * D / 4;   // float4 columns of a run's output
+    static constexpr int NC = G * D / 4 / CS;  // float4 columns of a CTA: a CS-th of a run's output
     static constexpr int NCT = NC / CPT;   // threads of a group
     static constexpr int MAX_THREADS = CPT == 1 ? kCombineMaxThreads : NCT;
     static constexpr int MIN_CTAS = CPT == 1 ? 1 : 28 / ((NCT + 31) / 32);  // 28 warps an SM: 72 registers
@@ -1075,22 +1110,22 @@ struct CombineShape {
 };
 
 // shared memory of a CTA of `threads` threads: the groups' states for the
-// in-order merge (none with one group)
-template <int D, int G, int CPT>
+// merge (none with one group)
+template <int D, int G, int CPT, int CS>
 inline size_t combine_smem_bytes(int threads)
 {
-    return threads > CombineShape<D, G, CPT>::NCT ? (size_t)threads * CPT * (2 * sizeof(float) + sizeof(float4)) : 0;
+    return threads > CombineShape<D, G, CPT, CS>::NCT ? (size_t)threads * CPT * (2 * sizeof(float) + sizeof(float4)) : 0;
 }
 
-template <int D, int G, int CPT>
-__global__ void __launch_bounds__(CombineShape<D, G, CPT>::MAX_THREADS, CombineShape<D, G, CPT>::MIN_CTAS)
+template <int D, int G, int CPT, int CS>
+__global__ void __launch_bounds__(CombineShape<D, G, CPT, CS>::MAX_THREADS, CombineShape<D, G, CPT, CS>::MIN_CTAS)
 combine_kernel(const __grid_constant__ CombineArgs c)
 {
-    using CS = CombineShape<D, G, CPT>;
+    using Sh = CombineShape<D, G, CPT, CS>;
     constexpr uint32_t MF = merge_floats<D, G>();
-    constexpr int NCT = CS::NCT;
-    constexpr int B = CS::BATCH;
-    static_assert(CS::NC % CPT == 0 && NCT <= kCombineMaxThreads, "whole columns per thread");
+    constexpr int NCT = Sh::NCT;
+    constexpr int B = Sh::BATCH;
+    static_assert(Sh::NC % CPT == 0 && NCT <= kCombineMaxThreads, "whole columns per thread");
     const int NG = (int)blockDim.x / NCT;  // groups of NCT threads
     extern __shared__ float4 s_dyn[];      // [CPT][blockDim] O, then M, then L (when NG > 1)
     const int r = blockIdx.x;
@@ -1112,7 +1147,7 @@ combine_kernel(const __grid_constant__ CombineArgs c)
     int col[CPT], h[CPT];
 #pragma unroll
     for (int j = 0; j < CPT; ++j) {
-        col[j] = tid % NCT + j * NCT;
+        col[j] = (int)blockIdx.y * Sh::NC + tid % NCT + j * NCT;
         h[j] = (col[j] * 4) / D;
     }
     // online merge of this group's records per column: M running max, L and
@@ -1147,58 +1182,37 @@ combine_kernel(const __grid_constant__ CombineArgs c)
 #pragma unroll
         for (int b = 0; b < B; ++b)
 #pragma unroll
-            for (int j = 0; j < CPT; ++j) {
-                if (mv[b][j] == -INFINITY) continue;  // past the run's records
-                const float Mn = fmaxf(M[j], mv[b][j]);
-                const float sa = fast_exp2(M[j] - Mn), sb = fast_exp2(mv[b][j] - Mn);
-                L[j] = L[j] * sa + lv[b][j] * sb;
-                O[j].x = O[j].x * sa + ov[b][j].x * sb;
-                O[j].y = O[j].y * sa + ov[b][j].y * sb;
-                O[j].z = O[j].z * sa + ov[b][j].z * sb;
-                O[j].w = O[j].w * sa + ov[b][j].w * sb;
-                M[j] = Mn;
-            }
+            for (int j = 0; j < CPT; ++j)
+                merge_record(M[j], L[j], O[j], mv[b][j], lv[b][j], ov[b][j]);
     }
     if (NG > 1) {
         const int nt = (int)blockDim.x;
         float4 *s_O = s_dyn;
         float *s_M = reinterpret_cast<float *>(s_dyn + CPT * nt);
         float *s_L = s_M + CPT * nt;
+        // halves of the groups in turn: group q takes in group q + half
+        for (int n = NG; n > 1;) {
+            const int half = (n + 1) / 2;
+            if (grp >= half && grp < n)
 #pragma unroll
-        for (int j = 0; j < CPT; ++j) {
-            s_M[j * nt + tid] = M[j];
-            s_L[j * nt + tid] = L[j];
-            s_O[j * nt + tid] = O[j];
+                for (int j = 0; j < CPT; ++j) {
+                    s_M[j * nt + tid] = M[j];
+                    s_L[j * nt + tid] = L[j];
+                    s_O[j * nt + tid] = O[j];
+                }
+            __syncthreads();
+            if (grp + half < n)
+#pragma unroll
+                for (int j = 0; j < CPT; ++j) {
+                    const int i = j * nt + tid + half * NCT;
+                    merge_record(M[j], L[j], O[j], s_M[i], s_L[i], s_O[i]);
+                }
+            n = half;
         }
-        __syncthreads();
         if (grp != 0) return;
-        // merge the groups in order
-        for (int q = 1; q < NG; ++q)
-#pragma unroll
-            for (int j = 0; j < CPT; ++j) {
-                const int i = j * nt + tid + q * NCT;
-                const float mq = s_M[i];
-                if (mq == -INFINITY) continue;  // group had no records
-                const float Mn = fmaxf(M[j], mq);
-                const float sa = fast_exp2(M[j] - Mn), sb = fast_exp2(mq - Mn);
-                const float4 oq = s_O[i];
-                L[j] = L[j] * sa + s_L[i] * sb;
-                O[j].x = O[j].x * sa + oq.x * sb;
-                O[j].y = O[j].y * sa + oq.y * sb;
-                O[j].z = O[j].z * sa + oq.z * sb;
-                O[j].w = O[j].w * sa + oq.w * sb;
-                M[j] = Mn;
-            }
     }
 #pragma unroll
-    for (int j = 0; j < CPT; ++j) {
-        __nv_bfloat162 lo = __floats2bfloat162_rn(O[j].x / L[j], O[j].y / L[j]);
-        __nv_bfloat162 hi = __floats2bfloat162_rn(O[j].z / L[j], O[j].w / L[j]);
-        uint2 w2;
-        w2.x = *reinterpret_cast<uint32_t *>(&lo);
-        w2.y = *reinterpret_cast<uint32_t *>(&hi);
-        *reinterpret_cast<uint2 *>(orow + col[j] * 4) = w2;
-    }
+    for (int j = 0; j < CPT; ++j) store_column(orow + col[j] * 4, O[j], L[j]);
 }
 
 // host helpers ---------------------------------------------------------------

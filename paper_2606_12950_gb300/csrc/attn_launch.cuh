@@ -46,6 +46,19 @@ int cached_occupancy(Fn fn, int threads, size_t smem, int *occ, OccCache &c)
     return KV_OK;
 }
 
+// The combine over c's runs: `groups` thread groups a CTA, CS CTAs a run.
+template <int D, int G, int CPT, int CS>
+int combine_launch(const CombineArgs &c, int groups, cudaLaunchConfig_t cfg)
+{
+    const int threads = groups * CombineShape<D, G, CPT, CS>::NCT;
+    cfg.gridDim = dim3((unsigned)(c.S * c.Hkv), (unsigned)CS);
+    cfg.blockDim = dim3((unsigned)threads);
+    cfg.dynamicSmemBytes = combine_smem_bytes<D, G, CPT, CS>(threads);
+    if (cudaLaunchKernelEx(&cfg, combine_kernel<D, G, CPT, CS>, c) != cudaSuccess) return KV_ERR_CUDA;
+    kvp_note_stream(cfg.stream, true);
+    return KV_OK;
+}
+
 // what: kLaunchQuery (only *P_out), kLaunchBoth (attention, then combine),
 // kLaunchAttention, kLaunchCombine
 enum { kLaunchQuery = 0, kLaunchBoth = 1, kLaunchAttention = 2, kLaunchCombine = 3 };
@@ -92,28 +105,19 @@ int attn_run(const CUtensorMap *tmap, AttnArgs a, int P_req, int sm_count, cudaS
     if (what == kLaunchAttention) return KV_OK;
     CombineArgs c{a.out, a.ws_run, a.ws_part, a.S, a.Hkv, a.skip, a.ws_pre, a.KS};
     cudaLaunchConfig_t ccfg = cfg;
-    // records per run: at most P * nwarps parts spread over the runs, plus
-    // the prefix records in shared-prefix mode
-    const double per_run = (double)P * a.nwarps / std::max(1, a.S * a.Hkv) + 1.0 + (a.skip ? a.KS : 0);
-    const int groups = combine_groups<D, G>(per_run, a.skip != nullptr);
-    ccfg.gridDim = dim3((unsigned)(a.S * a.Hkv));
+    // records per run: at most one per part, spread over the runs, plus the
+    // prefix records in shared-prefix mode
+    const int runs = a.S * a.Hkv;
+    const double per_run = (double)P * a.nwarps / std::max(1, runs) + 1.0 + (a.skip ? a.KS : 0);
     if constexpr (G * D / 4 >= 128) {
         // one group in shared-prefix mode: two columns a thread, so that
         // every member run fits in one wave
-        if (groups == 1 && a.skip != nullptr) {
-            ccfg.blockDim = dim3((unsigned)CombineShape<D, G, 2>::NCT);
-            ccfg.dynamicSmemBytes = 0;
-            if (cudaLaunchKernelEx(&ccfg, combine_kernel<D, G, 2>, c) != cudaSuccess) return KV_ERR_CUDA;
-            kvp_note_stream(st, true);
-            return KV_OK;
-        }
+        if (a.skip != nullptr && combine_groups<D, G, 1>(per_run) == 1) return combine_launch<D, G, 2, 1>(c, 1, ccfg);
     }
-    const int threads = groups * (G * D / 4);
-    ccfg.blockDim = dim3((unsigned)threads);
-    ccfg.dynamicSmemBytes = combine_smem_bytes<D, G, 1>(threads);
-    if (cudaLaunchKernelEx(&ccfg, combine_kernel<D, G, 1>, c) != cudaSuccess) return KV_ERR_CUDA;
-    kvp_note_stream(st, true);
-    return KV_OK;
+    // few runs: each run's columns spread over CS CTAs (kSlicedCtas)
+    if (8 * runs <= kSlicedCtas * sm_count) return combine_launch<D, G, 1, 8>(c, combine_groups<D, G, 8>(per_run), ccfg);
+    if (4 * runs <= kSlicedCtas * sm_count) return combine_launch<D, G, 1, 4>(c, combine_groups<D, G, 4>(per_run), ccfg);
+    return combine_launch<D, G, 1, 1>(c, combine_groups<D, G, 1>(per_run), ccfg);
 }
 
 // Shared-prefix kernel: with launch = false only reports the CTAs that fit

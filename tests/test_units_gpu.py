@@ -68,3 +68,34 @@ def test_context_lengths_at_box_and_unit_edges(d, bs, variant, fused):
     assert np.array_equal(pool.download(), ref_pool)
     _check(db.out_f64(), oracle.batch_attention(b, pool=ref_pool), (d, bs, variant, fused))
     assert pool.error() == 0
+
+
+def _attend(b, max_blocks=None):
+    """Fused append + attention of batch b, its table widened to max_blocks."""
+    from paper_2606_12950_gb300.runner import DeviceBatch, DevicePool
+
+    if max_blocks is not None:
+        wide = np.full((b.S, max_blocks), -1, np.int32)
+        wide[:, : b.max_blocks] = b.table
+        b.table, b.max_blocks = wide, max_blocks
+    pool = DevicePool(b.n_pages, b.page_elems * 2, b.bs, [(b.Hkv, b.d)])
+    pool.upload(b.pool)
+    db = DeviceBatch(pool, 0, b)
+    db.append_attend()
+    torch.cuda.synchronize()
+    assert pool.error() == 0
+    return pool, db
+
+
+@pytest.mark.parametrize("G,d", [(1, 64), (4, 128), (5, 64), (8, 128)])
+@pytest.mark.parametrize("S", [1, 2, 76, 77, 152, 153])
+def test_combine_with_few_and_many_runs(S, G, d):
+    """One KV head, so S runs: either side of the lines at which the combine
+    spreads a run's columns over 8, 4 or 1 CTAs (152 SMs), with runs of one
+    record and of several hundred."""
+    lens = [5000 if S < 3 else 700] + [17 + 41 * s % 333 for s in range(1, S)]
+    b = W.make_batch(7100 + S + G, lens, Hq=G, Hkv=1, d=d, bs=16, extra_blocks=3)
+    pool, db = _attend(b)
+    ref_pool = oracle.batch_append(b)
+    assert np.array_equal(pool.download(), ref_pool)
+    _check(db.out_f64(), oracle.batch_attention(b, pool=ref_pool), (S, G, d))
