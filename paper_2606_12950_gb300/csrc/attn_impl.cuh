@@ -33,6 +33,21 @@
 // that ends inside a warp's range is written out by that warp directly; no
 // state is merged between warps of a CTA.
 //
+// Small batches (MERGE, chosen by attn_run): a part is a CTA's range of units,
+// cut again into one range per warp.  What bounds them is latency: a warp
+// takes its units one after another, and each part's record is one more for
+// the combine to fetch.  So the units go to as many warps as there are (one
+// unit a warp at least, instead of 64 tokens), and the warps of a CTA that
+// share a run merge their states in shared memory: the CTA leaves the run's
+// output, or one record for the combine instead of six.  One sequence of 8193
+// tokens (32 q / 8 KV heads, 33.6 MB) has 38 records a run instead of 128;
+// a step took 18.0 us before and 14.4 now (of it, the combine's column slices
+// below: 2.3); 8 sequences of 601-3500 tokens (40 q / 8 KV heads, 67 MB) 20.9
+// and 19.9.  The line at 8 units a warp: with the merge at every size the
+// 64-sequence batch (29 units a warp) took 72.9 us against 72.2, because
+// every CTA then waits for its slowest warp; at 4 units instead of 8 the 8
+// sequences (4.5 units a warp) took 21.1 us against 20.3.
+//
 // Grid-to-grid order: the kernel is launched as a programmatic dependent.
 // Alone it releases the next grid and waits for the one before; as part of
 // a chain (beside the shared-prefix kernel, or the later batches of several
@@ -87,6 +102,8 @@ constexpr int kSub = kUnit<D> / kTile;            // boxes' rows per unit
 // a part's least tokens (4 units at d = 128, 2 at d = 64): with 128 at d = 64
 // a step of four short sequences took 18.5 us instead of 15.5
 constexpr int kMinPartTokens = 64;
+// Below this many units a warp the parts are CTAs (MERGE): see the kernel.
+constexpr int kMergeUnits = 8;
 constexpr uint32_t kHalfBytes = kTile * 128;      // one 64-column box: 16 rows x 128 B
 constexpr uint64_t kWaitLimitNs = 2000000000ull;  // bounded mbarrier waits: 2 s
 
@@ -743,7 +760,7 @@ __device__ __forceinline__ void issue_half(const CUtensorMap *tmap, const AttnAr
                 tma_load_2d(dst + (j + h) * kHalfBytes, tmap, h * 64, y[j] + which * a.Hkv * a.bs, bar, policy);
 }
 
-template <int D, int G, class Comp>
+template <int D, int G, class Comp, bool MERGE>
 __global__ void __launch_bounds__(kThreads, Comp::kMinBlocks)
 paged_attn_kernel(const __grid_constant__ CUtensorMap tmap, const __grid_constant__ AttnArgs a)
 {
@@ -761,7 +778,9 @@ paged_attn_kernel(const __grid_constant__ CUtensorMap tmap, const __grid_constan
     uint8_t *stages = smem;                                                              // [NW][kStages][STAGE]
     uint8_t *qbufs = stages + (size_t)NW * kStages * STAGE_BYTES;                        // [NW][QB]
     uint8_t *abufs = qbufs + (size_t)NW * QB;                                            // [NW][AB]
-    uint64_t *bars = reinterpret_cast<uint64_t *>(abufs + (size_t)NW * AB);              // K[w][st], V[w][st]
+    uint8_t *mbufs = abufs + (size_t)NW * AB;                                            // [NW] records, with MERGE
+    int4 *chains = reinterpret_cast<int4 *>(mbufs + (MERGE ? (size_t)NW * MF * 4 : 0));  // [NW]
+    uint64_t *bars = reinterpret_cast<uint64_t *>(chains + (MERGE ? NW : 0));    // K[w][st], V[w][st]
     int32_t *misc = reinterpret_cast<int32_t *>(bars + 2 * NW * kStages);               // [16] scratch
     int32_t *T = misc + 16;                                                              // [S + 1]
     int32_t *NL = T + a.S + 1;                                                           // [S]
@@ -883,21 +902,23 @@ paged_attn_kernel(const __grid_constant__ CUtensorMap tmap, const __grid_constan
     }
 
     // The W units are cut into NP = min(P * NW, W) equal parts; part i is
-    // [i*W/NP, (i+1)*W/NP) and belongs to warp i % NW of CTA i / NW.
+    // [i*W/NP, (i+1)*W/NP) and belongs to warp i % NW of CTA i / NW (with
+    // MERGE to CTA i, at least NW units each).
     // With NP <= W every part is non-empty, so a run's contributors are
     // exactly the parts part_of(first unit) .. part_of(last unit).  A part
     // gets at least MIN_UNITS units when the batch is small (fewer
     // partials to write and merge; enough warps still stream to fill HBM).
     const int64_t W = T[S];
     constexpr int MIN_UNITS = kMinPartTokens / UNIT;
-    const int64_t np_min = W > 0 ? (W / MIN_UNITS > 0 ? W / MIN_UNITS : 1) : 0;
-    const int64_t NP = np_min < (int64_t)a.P * NW ? np_min : (int64_t)a.P * NW;
-    const int64_t first_part = (int64_t)blockIdx.x * NW;
+    const int64_t most = MERGE ? (int64_t)a.P : (int64_t)a.P * NW;
+    const int64_t fine = MERGE ? (W + NW - 1) / NW : W / MIN_UNITS > 0 ? W / MIN_UNITS : W;
+    const int64_t NP = fine < most ? fine : most;
+    const int64_t first_part = MERGE ? (int64_t)blockIdx.x : (int64_t)blockIdx.x * NW;
     if (first_part >= NP) {
         if (chained) grid_dependency_wait();
         return;
     }
-    const int64_t last_part = first_part + NW < NP ? first_part + NW : NP;  // exclusive
+    const int64_t last_part = MERGE ? first_part + 1 : first_part + NW < NP ? first_part + NW : NP;  // exclusive
     const int32_t cu0 = (int32_t)(first_part * W / NP);                             // this CTA's units
     const int32_t cu1 = (int32_t)(last_part * W / NP);
 
@@ -909,13 +930,22 @@ paged_attn_kernel(const __grid_constant__ CUtensorMap tmap, const __grid_constan
         __syncthreads();
     }
 
-    const int64_t part = first_part + warp;
-    if (part >= NP) {  // no CTA-wide barrier below this point
+    const int64_t part = MERGE ? first_part : first_part + warp;
+    if (part >= NP) {  // no CTA-wide barrier below this point without MERGE
         if (chained) grid_dependency_wait();
         return;
     }
-    const int32_t u0 = (int32_t)(part * W / NP);
-    const int32_t u1 = (int32_t)((part + 1) * W / NP);
+    // this warp's units [u0, u1), and its part's [g0, g1): the same without MERGE
+    const int32_t nu = cu1 - cu0;
+    const int32_t u0 = MERGE ? cu0 + warp * nu / NW : (int32_t)(part * W / NP);
+    const int32_t u1 = MERGE ? cu0 + (warp + 1) * nu / NW : (int32_t)((part + 1) * W / NP);
+    const int32_t g0 = MERGE ? cu0 : u0, g1 = MERGE ? cu1 : u1;
+    float *mbuf = reinterpret_cast<float *>(mbufs) + (size_t)warp * MF;
+    if (MERGE && lane == 0) {
+        chains[warp].x = -1;
+        if (u0 == u1)  // no units: nothing to merge from this warp
+            for (int h = 0; h < G; ++h) mbuf[G * D + h] = -INFINITY;
+    }
 
     const uint64_t policy = l2_policy_evict_first();
     // stage st of this warp: its K and V tiles and their barriers
@@ -937,9 +967,9 @@ paged_attn_kernel(const __grid_constant__ CUtensorMap tmap, const __grid_constan
     uint8_t *ab = abufs + (size_t)warp * AB;
     const uint32_t qb_addr = smem_u32(qb), ab_addr = smem_u32(ab);
     {
-        const int s0 = find_seq(T, S, u0);
+        const int s0 = find_seq(T, S, MERGE && u0 == u1 ? cu0 : u0);
         const int32_t nt0 = (T[s0 + 1] - T[s0]) / Hkv;
-        const uint16_t *src = a.q + ((int64_t)s0 * Hq + (int64_t)((u0 - T[s0]) / nt0) * G) * D;
+        const uint16_t *src = a.q + ((int64_t)s0 * Hq + (int64_t)(((MERGE && u0 == u1 ? cu0 : u0) - T[s0]) / nt0) * G) * D;
         for (uint32_t c = lane; c < QB / 16; c += 32) cp_async16(qb_addr + c * 16, src + c * 8);
         cp_async_commit();
     }
@@ -1028,11 +1058,54 @@ paged_attn_kernel(const __grid_constant__ CUtensorMap tmap, const __grid_constan
         const bool split = p_first != p_last || pc.skip > 0;
         uint16_t *orow = a.out + ((int64_t)pc.s * Hq + (int64_t)pc.g * G) * D;
         float *slot = a.ws_part + ((int64_t)r + part) * MF;
-        make_ready();
-        comp.store(orow, slot, split, lane);
-        if (part == p_first && lane == 0)  // each run has one first part: it tells the combine
-            a.ws_run[r] = make_int2(p_first, split ? p_last - p_first + 1 : 0);
+        // (MERGE) the part's share of the run; it may go on over several warps
+        const int32_t lo = pc.run_begin > g0 ? pc.run_begin : g0, hi = pc.run_end < g1 ? pc.run_end : g1;
+        if (!MERGE || (pc.pb == lo && pc.pe == hi)) {
+            make_ready();
+            comp.store(orow, slot, split, lane);
+            if (part == p_first && lane == 0)  // each run has one first part: it tells the combine
+                a.ws_run[r] = make_int2(p_first, split ? p_last - p_first + 1 : 0);
+        } else if (pc.pb != lo) {  // goes on from an earlier warp, whose chain merges it
+            comp.store(nullptr, mbuf, true, lane);
+        } else {  // goes on in the next warp: the last piece here, so the stage is free
+            comp.store(nullptr, reinterpret_cast<float *>(wstage), true, lane);
+            if (lane == 0)
+                chains[warp] = make_int4(r, (int)(((int64_t)(hi - cu0) * NW - 1) / nu) - warp, p_first,
+                                         split ? p_last - p_first + 1 : 0);
+        }
         u = pc.pe;
+    }
+    if constexpr (MERGE) {
+        __syncthreads();
+        // CTA-level merge: chain w is the run whose share of this CTA starts in
+        // warp w and goes on through warp w + chains[w].y; its states (base-2
+        // online softmax) are merged in warp order, one thread per float4
+        // column, into the output (a run inside this CTA) or one record
+        constexpr int NC = G * D / 4;
+        for (int i = tid; i < NW * NC; i += NT) {
+            const int w = i / NC, c = i % NC, h = c * 4 / D;
+            const int4 ch = chains[w];
+            if (ch.x < 0) continue;
+            float M = -INFINITY, L = 0.f;
+            float4 O = make_float4(0.f, 0.f, 0.f, 0.f);
+            for (int k = 0; k <= ch.y; ++k) {
+                const float *rec = k == 0 ? reinterpret_cast<const float *>(stages + (size_t)w * kStages * STAGE_BYTES)
+                                          : reinterpret_cast<const float *>(mbufs) + (size_t)(w + k) * MF;
+                merge_record(M, L, O, rec[G * D + h], rec[G * D + G + h], *reinterpret_cast<const float4 *>(rec + c * 4));
+            }
+            make_ready();
+            if (ch.w == 0) {
+                store_column(a.out + (int64_t)ch.x * (G * D) + c * 4, O, L);
+            } else {
+                float *slot = a.ws_part + ((int64_t)ch.x + part) * MF;
+                *reinterpret_cast<float4 *>(slot + c * 4) = O;
+                if (c * 4 % D == 0) {
+                    slot[G * D + h] = M;
+                    slot[G * D + G + h] = L;
+                }
+            }
+            if (c == 0 && ch.z == (int)part) a.ws_run[ch.x] = make_int2(ch.z, ch.w);
+        }
     }
     if (chained) grid_dependency_wait();
 }
@@ -1190,10 +1263,12 @@ combine_kernel(const __grid_constant__ CombineArgs c)
         float4 *s_O = s_dyn;
         float *s_M = reinterpret_cast<float *>(s_dyn + CPT * nt);
         float *s_L = s_M + CPT * nt;
-        // halves of the groups in turn: group q takes in group q + half
+        // the first `to` groups take in the others, half of them at a time
+        // while there are more than four (a barrier a round costs more than
+        // merging three states)
         for (int n = NG; n > 1;) {
-            const int half = (n + 1) / 2;
-            if (grp >= half && grp < n)
+            const int to = n <= 4 ? 1 : (n + 1) / 2;
+            if (grp >= to && grp < n)
 #pragma unroll
                 for (int j = 0; j < CPT; ++j) {
                     s_M[j * nt + tid] = M[j];
@@ -1201,13 +1276,14 @@ combine_kernel(const __grid_constant__ CombineArgs c)
                     s_O[j * nt + tid] = O[j];
                 }
             __syncthreads();
-            if (grp + half < n)
+            if (grp < to)
+                for (int q = to; grp + q < n; q += to)
 #pragma unroll
-                for (int j = 0; j < CPT; ++j) {
-                    const int i = j * nt + tid + half * NCT;
-                    merge_record(M[j], L[j], O[j], s_M[i], s_L[i], s_O[i]);
-                }
-            n = half;
+                    for (int j = 0; j < CPT; ++j) {
+                        const int i = j * nt + tid + q * NCT;
+                        merge_record(M[j], L[j], O[j], s_M[i], s_L[i], s_O[i]);
+                    }
+            n = to;
         }
         if (grp != 0) return;
     }
@@ -1219,10 +1295,10 @@ combine_kernel(const __grid_constant__ CombineArgs c)
 constexpr int kRowsCap = 2048;
 
 template <int D, int G>
-inline size_t attn_smem_bytes(int S, int rows_cap, int nwarps)
+inline size_t attn_smem_bytes(int S, int rows_cap, int nwarps, bool merge)
 {
     const size_t stage = 2ull * (D / 64) * kSub<D> * kHalfBytes;
-    const size_t bufs = (size_t)G * D * 2 + 2 * D * 2;  // per warp: q rows, new K/V rows
+    const size_t bufs = (size_t)G * D * 2 + 2 * D * 2 + (merge ? merge_floats<D, G>() * 4 + 16 : 0);  // per warp: q rows, new K/V rows; a record, its chain
     return 1024 + (size_t)nwarps * (kStages * stage + bufs) + (2 * nwarps * kStages) * 8 + 64 + (size_t)(3 * S + 1) * 4 +
            (size_t)rows_cap * 4;
 }

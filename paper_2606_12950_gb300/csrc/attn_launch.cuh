@@ -66,16 +66,18 @@ enum { kLaunchQuery = 0, kLaunchBoth = 1, kLaunchAttention = 2, kLaunchCombine =
 template <int D, int G, class Comp>
 int attn_run(const CUtensorMap *tmap, AttnArgs a, int P_req, int sm_count, cudaStream_t st, int what, int *P_out)
 {
-    auto fn = paged_attn_kernel<D, G, Comp>;
+    auto fn = paged_attn_kernel<D, G, Comp, false>;
+    auto fn_merge = paged_attn_kernel<D, G, Comp, true>;
     static std::atomic<bool> attr_set{false};
     if (!attr_set.load()) {
-        if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemMax) != cudaSuccess)
+        if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemMax) != cudaSuccess ||
+            cudaFuncSetAttribute(fn_merge, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemMax) != cudaSuccess)
             return KV_ERR_CUDA;
         attr_set.store(true);
     }
     // six warps a CTA, eight beside the shared-prefix kernel (kPlainWarps)
     a.nwarps = a.skip != nullptr ? kWarps : kPlainWarps;
-    const size_t smem = attn_smem_bytes<D, G>(a.S, kRowsCap, a.nwarps);
+    size_t smem = attn_smem_bytes<D, G>(a.S, kRowsCap, a.nwarps, false);
     if (smem > kSmemMax) return KV_ERR_INVALID_ARG;  // S too large for the per-CTA sequence index
     int occ = 0;
     static OccCache occ_cache;
@@ -85,6 +87,27 @@ int attn_run(const CUtensorMap *tmap, AttnArgs a, int P_req, int sm_count, cudaS
     if (what == kLaunchQuery) return KV_OK;
     a.rows_cap = kRowsCap;
     a.P = P;
+    // A batch whose table has room for fewer than kMergeUnits units a warp
+    // runs with its CTAs as the parts (MERGE), if the merge's buffers cost no
+    // CTA per SM.  The rule sees the table's width, not the lengths, so that
+    // a call gives the same bits whether the lengths come with it or not.
+    int parts_per_cta = a.nwarps;
+    const int64_t most_units =
+        (int64_t)a.S * a.Hkv * (((int64_t)a.max_blocks * a.bs + kUnit<D> - 1) / kUnit<D>);
+    if (most_units < (int64_t)kMergeUnits * P * a.nwarps) {
+        const size_t smem_merge = attn_smem_bytes<D, G>(a.S, kRowsCap, a.nwarps, true);
+        int occ_merge = 0;
+        static OccCache merge_cache;
+        if (smem_merge <= kSmemMax) {
+            if (cached_occupancy(fn_merge, a.nwarps * 32, smem_merge, &occ_merge, merge_cache) != KV_OK)
+                return KV_ERR_CUDA;
+            if (occ_merge >= occ) {
+                fn = fn_merge;
+                smem = smem_merge;
+                parts_per_cta = 1;
+            }
+        }
+    }
     // both kernels are programmatic dependents of what precedes them in the
     // stream: they may be scheduled early and wait on the device
     // (griddepcontrol.wait) for the previous grid to complete
@@ -108,7 +131,7 @@ int attn_run(const CUtensorMap *tmap, AttnArgs a, int P_req, int sm_count, cudaS
     // records per run: at most one per part, spread over the runs, plus the
     // prefix records in shared-prefix mode
     const int runs = a.S * a.Hkv;
-    const double per_run = (double)P * a.nwarps / std::max(1, runs) + 1.0 + (a.skip ? a.KS : 0);
+    const double per_run = (double)P * parts_per_cta / std::max(1, runs) + 1.0 + (a.skip ? a.KS : 0);
     if constexpr (G * D / 4 >= 128) {
         // one group in shared-prefix mode: two columns a thread, so that
         // every member run fits in one wave

@@ -99,3 +99,57 @@ def test_combine_with_few_and_many_runs(S, G, d):
     ref_pool = oracle.batch_append(b)
     assert np.array_equal(pool.download(), ref_pool)
     _check(db.out_f64(), oracle.batch_attention(b, pool=ref_pool), (S, G, d))
+
+
+MERGE_LENS = {
+    "one_token": [0],
+    "under_a_warp": [15, 40],
+    "many_short": [1 + 37 * s % 90 for s in range(40)],
+    "one_long": [5000],
+    "long_and_short": [3000, 5, 700, 31, 1, 2047, 16, 64],
+}
+
+
+@pytest.mark.parametrize("lens", MERGE_LENS.values(), ids=MERGE_LENS.keys())
+@pytest.mark.parametrize("G,Hkv,d", [(1, 4, 128), (4, 8, 128), (8, 1, 128), (5, 2, 64), (4, 8, 64)])
+def test_cta_level_parts_against_the_oracle_and_the_general_path(G, Hkv, d, lens):
+    """A small batch merges its warps' records inside each CTA; the same batch
+    with a table too wide for that takes the general path.  Both against the
+    oracle, and against each other.  The two paths round a token's weight to
+    bf16 against different running maxima, 2^-9 of it at most on each side, so
+    they differ by at most 2 * 2^-9 * sum(p |v|) <= 2^-8 max|v|, and by the
+    outputs' own rounding, 2^-9 |out| on each side (the fp32 sums add less
+    than 2^-16 of that)."""
+    outs = []
+    for width in (None, 16384):
+        b = W.make_batch(7200 + G + d, lens, Hq=G * Hkv, Hkv=Hkv, d=d, bs=16, extra_blocks=3)
+        _nan_past_contexts(b)
+        pool, db = _attend(b, width)
+        ref_pool = oracle.batch_append(b)
+        assert np.array_equal(pool.download(), ref_pool)
+        outs.append(db.out_f64())
+        _check(outs[-1], oracle.batch_attention(b, pool=ref_pool), (G, Hkv, d, width))
+    vals = W.bf16_bits_to_f64(ref_pool)
+    vmax = np.abs(vals[np.isfinite(vals)]).max()
+    assert np.all(np.abs(outs[0] - outs[1]) <= 2.0 ** -8 * (vmax + np.abs(outs[1])))
+
+
+def test_cta_level_parts_with_a_shared_prefix():
+    """Short suffixes beside the prefix kernel: every member leaves a record,
+    also where its suffix lies inside one CTA."""
+    from paper_2606_12950_gb300 import kvpool as K
+    from paper_2606_12950_gb300.runner import DeviceBatch, DevicePool
+
+    pre = [256 + n for n in (0, 3, 16, 47, 300, 64)] + [90, 33]
+    groups = [(list(range(6)), 256)]
+    b = W.make_batch(7300, pre, Hq=8, Hkv=2, d=128, bs=16, extra_blocks=3)
+    W.share_prefix(b, groups)
+    pool = DevicePool(b.n_pages, b.page_elems * 2, b.bs, [(b.Hkv, b.d)])
+    pool.upload(b.pool)
+    db = DeviceBatch(pool, 0, b)
+    db.cascade(K.PrefixPlan(groups))
+    torch.cuda.synchronize()
+    ref_pool = oracle.batch_append(b)
+    assert np.array_equal(pool.download(), ref_pool)
+    _check(db.out_f64(), oracle.batch_attention(b, pool=ref_pool), "prefix")
+    assert pool.error() == 0
