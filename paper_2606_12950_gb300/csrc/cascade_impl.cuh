@@ -11,7 +11,15 @@
 //   S = Q K^T     tcgen05.mma, M = 128 query rows, N = 128 keys, fp32 in TMEM
 //   softmax       one thread per row, S read from TMEM, base 2, lazy rescale
 //   O += P V      tcgen05.mma, P (bf16) from TMEM, V from shared memory, O in TMEM
-// with 128-key K/V tiles streamed by TMA through a 2-stage ring.  The
+// with 128-key K/V tiles streamed by TMA through a 2-stage ring.  Beside the
+// suffix stream, which keeps HBM's queues full, a tile's loads take several
+// microseconds, longer than the tensor work on the tile before: so K and V of
+// a stage are released and reloaded apart (K as soon as the tile's scores are
+// done), and the producer asks L2 for the tiles kPreAhead further on.  With
+// 4096-token prefixes of 3 groups (24 CTAs) beside 190 suffixes the step took
+// 135 us with one barrier a stage and no requests ahead (4.5 us a tile, 2.7
+// alone on the GPU) and 115 with both and the record stores of the epilogue;
+// 2 or 8 tiles ahead instead of 4: 116 and 116.  The
 // softmax writes P (bf16) back over S in TMEM, and the P.V MMA reads its A
 // operand from there, so P never touches shared memory.  A CTA holds two Q
 // tiles that share every K/V tile: while one tile's four warps run the
@@ -35,6 +43,7 @@ constexpr int kPreChunk = 64;             // granularity of prefix lengths and k
 constexpr int kPreStages = 2;
 constexpr int kPreSoftWarps = 4;          // per Q tile: one thread per query row
 constexpr int kPreThreads = (kPreQTiles * kPreSoftWarps + 2) * 32;  // + TMA warp + MMA warp
+constexpr int kPreAhead = 4;              // key tiles asked of L2 ahead of their loads
 constexpr int kPreRowsCap = 256;          // 16-token sub-tiles resolved up front
 constexpr int kMaxKeySplits = 8;
 constexpr int kCascadeWords = 4080;       // most plan words (the plan kernel's parameters, then the workspace)
@@ -101,8 +110,9 @@ struct PreSmem {
     static constexpr uint32_t Q_OFF = 0;
     static constexpr uint32_t ST_OFF = kPreQTiles * Q_TILE;
     static constexpr uint32_t BAR_OFF = ST_OFF + kPreStages * STAGE;
-    // full, empty per stage; per Q tile: s_full, p_full, o_done; fin; q_ready
-    static constexpr int NBARS = 2 * kPreStages + 3 * kPreQTiles + 2;
+    // full and empty per stage, of K and of V; per Q tile: s_full, p_full,
+    // o_done; fin; q_ready
+    static constexpr int NBARS = 4 * kPreStages + 3 * kPreQTiles + 2;
     static constexpr uint32_t SLOT_OFF = BAR_OFF + NBARS * 8;
     static constexpr uint32_t ROWS_OFF = SLOT_OFF + 16;
     static constexpr uint32_t BYTES = ROWS_OFF + kPreRowsCap * 4;
@@ -129,7 +139,8 @@ cascade_prefix_kernel(const __grid_constant__ CUtensorMap tmap, const __grid_con
     uint32_t *tslot = reinterpret_cast<uint32_t *>(smem + L::SLOT_OFF);
     int32_t *rows = reinterpret_cast<int32_t *>(smem + L::ROWS_OFF);
     auto bar = [&](int i) { return smem_u32(&bars[i]); };
-    constexpr int FULL = 0, EMPTY = kPreStages, QB = 2 * kPreStages, FIN = QB + 3 * kPreQTiles, Q_READY = FIN + 1;
+    constexpr int FULL_K = 0, EMPTY_K = kPreStages, FULL_V = 2 * kPreStages, EMPTY_V = 3 * kPreStages;
+    constexpr int QB = 4 * kPreStages, FIN = QB + 3 * kPreQTiles, Q_READY = FIN + 1;
     auto s_full = [&](int a) { return bar(QB + 3 * a); };
     auto p_full = [&](int a) { return bar(QB + 3 * a + 1); };
     auto o_done = [&](int a) { return bar(QB + 3 * a + 2); };
@@ -142,10 +153,7 @@ cascade_prefix_kernel(const __grid_constant__ CUtensorMap tmap, const __grid_con
     const int tile = bid / c.Hkv;
 
     if (tid == 0) {
-        for (int i = 0; i < kPreStages; ++i) {
-            mbar_init(bar(FULL + i), 1);
-            mbar_init(bar(EMPTY + i), 1);
-        }
+        for (int i = 0; i < 4 * kPreStages; ++i) mbar_init(bar(i), 1);
         for (int a = 0; a < kPreQTiles; ++a) {
             mbar_init(s_full(a), 1);
             mbar_init(p_full(a), kPreSoftWarps * 32);
@@ -183,14 +191,29 @@ cascade_prefix_kernel(const __grid_constant__ CUtensorMap tmap, const __grid_con
     const int32_t *mem_off = tile_off + c.n_groups + 1;
     const int32_t *tokens = mem_off + c.n_groups + 1;
     const int32_t *members = tokens + c.n_groups;
-    // (through L2: another kernel wrote the plan)
-    int grp = 0;
-    while (grp + 1 < c.n_groups && __ldcg(tile_off + grp + 1) <= tile) ++grp;
-    const int mo = __ldcg(mem_off + grp);
-    const int m0 = mo + (tile - __ldcg(tile_off + grp)) * MT;  // this CTA's members [m0, m1)
-    const int m1 = min(m0 + MT, __ldcg(mem_off + grp + 1));
+    // This CTA's group, member range and prefix, looked up by each warp: 32
+    // groups a round trip (through L2: another kernel wrote the plan; a
+    // round trip is 0.7 us, more beside the suffix stream, and the first loads
+    // wait for these).
+    int mo = 0, mend = 0, ntok = 0, tile0 = 0;
+    for (int i0 = 0; i0 < c.n_groups; i0 += 32) {
+        const int i = min(i0 + lane, c.n_groups - 1);
+        const int t_a = __ldcg(tile_off + i), t_b = __ldcg(tile_off + i + 1);
+        const int m_a = __ldcg(mem_off + i), m_b = __ldcg(mem_off + i + 1), tk = __ldcg(tokens + i);
+        const unsigned hit = __ballot_sync(0xffffffffu, t_b > tile);
+        if (hit) {
+            const int l = __ffs((int)hit) - 1;
+            tile0 = __shfl_sync(0xffffffffu, t_a, l);  // the group's first row tile
+            mo = __shfl_sync(0xffffffffu, m_a, l);
+            mend = __shfl_sync(0xffffffffu, m_b, l);
+            ntok = __shfl_sync(0xffffffffu, tk, l);
+            break;
+        }
+    }
     const int lead = __ldcg(members + mo);
-    const int ch_all = __ldcg(tokens + grp) / kPreChunk;        // 64-key chunks of the prefix
+    const int m0 = mo + (tile - tile0) * MT;                    // this CTA's members [m0, m1)
+    const int m1 = min(m0 + MT, mend);
+    const int ch_all = ntok / kPreChunk;                        // 64-key chunks of the prefix
     const int ch0 = ks * ch_all / c.KS, ch1 = (ks + 1) * ch_all / c.KS;  // non-empty: KS <= ch_all
     const int nch = ch1 - ch0;
     const int nt = (nch + 1) / 2;                                // key tiles; the last may hold one chunk
@@ -230,45 +253,53 @@ cascade_prefix_kernel(const __grid_constant__ CUtensorMap tmap, const __grid_con
         const uint64_t pol = l2_policy_evict_normal();  // the prefix is re-read by every row tile
         constexpr int NBOX = NSUB * HALVES;               // boxes of K (and of V) per full key tile
         static_assert(2 * NBOX <= 32, "one box per lane");
+        // box (j, h): rows 16j .. 16j + 15, columns 64h .. 64h + 63 of K
+        // (lanes below NBOX) or V (from NBOX on) of a key tile
+        const bool is_v = lane >= NBOX;
+        const int j = (lane % NBOX) / HALVES, h = (lane % NBOX) % HALVES;
+        auto row_of = [&](int t) {  // of this lane's box in key tile t: -1 outside the pool
+            const int32_t q = t * NSUB + j;
+            const int32_t y = q < kPreRowsCap ? rows[q] : pre_sub_row(c, lead, g, ch0 * CSUB + q);
+            return y < 0 ? y : y + (is_v ? c.Hkv * c.bs : 0);
+        };
+        auto mine_of = [&](int t) { return lane < 2 * NBOX && t < nt && j < tile_keys(t) / kTile; };
         for (int t = 0; t < nt; ++t) {
             const int st = t % kPreStages;
-            if (t >= kPreStages) wait_phase(bar(EMPTY + st), (uint32_t)(t / kPreStages - 1) & 1u, c.err, dead);
+            const uint32_t par = (uint32_t)(t / kPreStages - 1) & 1u;
             const int vsub = tile_keys(t) / kTile;        // sub-tiles loaded this tile
-            const uint32_t kdst = sbase + L::ST_OFF + st * L::STAGE, vdst = kdst + L::KV_TILE;
-            const int box = lane % NBOX, j = box / HALVES, h = box % HALVES;
-            const bool mine = lane < 2 * NBOX && j < vsub;
-            int32_t y = 0;
-            bool ok = true;
-            if (mine) {
-                const int32_t q = t * NSUB + j;
-                y = q < kPreRowsCap ? rows[q] : pre_sub_row(c, lead, g, ch0 * CSUB + q);
-                ok = y >= 0;
+            const bool mine = mine_of(t);
+            const int32_t y = mine ? row_of(t) : 0;
+            const bool ok = __all_sync(0xffffffffu, y >= 0);
+            if (!ok && lane == 0) report(c.err, KV_ERR_DEVICE_BOUNDS);
+            // the tile kPreAhead further on, into L2
+            if (mine_of(t + kPreAhead)) {
+                const int32_t ya = row_of(t + kPreAhead);
+                if (ya >= 0) tma_prefetch_2d(&tmap, h * 64, ya);
             }
-            ok = __all_sync(0xffffffffu, ok);
-            if (!ok) {
+            const uint32_t dst = sbase + L::ST_OFF + st * L::STAGE + (is_v ? L::KV_TILE : 0) + h * L::KV_HALF +
+                                 j * (kTile * 128);
+#pragma unroll
+            for (int kv = 0; kv < 2; ++kv) {
+                const uint32_t full = bar((kv ? FULL_V : FULL_K) + st);
+                if (t >= kPreStages) wait_phase(bar((kv ? EMPTY_V : EMPTY_K) + st), par, c.err, dead);
                 if (lane == 0) {
-                    report(c.err, KV_ERR_DEVICE_BOUNDS);
-                    mbar_arrive(bar(FULL + st));  // complete the phase without data
+                    if (ok)
+                        mbar_arrive_expect_tx(full, (uint32_t)vsub * HALVES * (kTile * 128));
+                    else
+                        mbar_arrive(full);  // complete the phase without data
                 }
                 __syncwarp();
-                continue;
-            }
-            if (lane == 0) mbar_arrive_expect_tx(bar(FULL + st), 2u * vsub * HALVES * (kTile * 128));
-            __syncwarp();
-            if (mine) {
-                const uint32_t off = h * L::KV_HALF + j * (kTile * 128);
-                if (lane < NBOX)
-                    tma_load_2d(kdst + off, &tmap, h * 64, y, bar(FULL + st), pol);
-                else
-                    tma_load_2d(vdst + off, &tmap, h * 64, y + c.Hkv * c.bs, bar(FULL + st), pol);
+                if (ok && mine && is_v == (kv == 1)) tma_load_2d(dst, &tmap, h * 64, y, full, pol);
             }
             __syncwarp();
         }
         // drain: the last stages' loads have landed (already waited on by the
         // MMA thread unless a wait ran out)
         if (lane == 0)
-            for (int t = max(0, nt - kPreStages); t < nt; ++t)
-                wait_phase(bar(FULL + t % kPreStages), (uint32_t)(t / kPreStages) & 1u, c.err, dead);
+            for (int t = max(0, nt - kPreStages); t < nt; ++t) {
+                wait_phase(bar(FULL_K + t % kPreStages), (uint32_t)(t / kPreStages) & 1u, c.err, dead);
+                wait_phase(bar(FULL_V + t % kPreStages), (uint32_t)(t / kPreStages) & 1u, c.err, dead);
+            }
     } else if (warp == MMA_WARP && lane == 0) {
         // ---- MMA issuer.  Per Q tile a and key tile t: S_a = Q_a K_t^T into
         // TMEM, then, once the tile's warps have written P (bf16) over S,
@@ -298,21 +329,25 @@ cascade_prefix_kernel(const __grid_constant__ CUtensorMap tmap, const __grid_con
             umma_commit(o_done(a));
         };
         wait_phase(bar(Q_READY), 0u, c.err, dead);
-        wait_phase(bar(FULL + 0), 0u, c.err, dead);
+        wait_phase(bar(FULL_K + 0), 0u, c.err, dead);
         tc_fence_after();
         for (int a = 0; a < kPreQTiles; ++a) issue_s(a, 0);
+        umma_commit(bar(EMPTY_K + 0));
         for (int t = 0; t < nt; ++t) {
             const bool next = t + 1 < nt;
             for (int a = 0; a < kPreQTiles; ++a) {
+                if (a == 0)
+                    wait_phase(bar(FULL_V + t % kPreStages), (uint32_t)(t / kPreStages) & 1u, c.err, dead);
                 wait_phase(p_full(a), (uint32_t)t & 1u, c.err, dead);
                 tc_fence_after();
                 issue_pv(a, t);
-                if (a == kPreQTiles - 1) umma_commit(bar(EMPTY + t % kPreStages));
+                if (a == kPreQTiles - 1) umma_commit(bar(EMPTY_V + t % kPreStages));
                 if (next) {
-                    if (a == 0) wait_phase(bar(FULL + (t + 1) % kPreStages), (uint32_t)((t + 1) / kPreStages) & 1u,
+                    if (a == 0) wait_phase(bar(FULL_K + (t + 1) % kPreStages), (uint32_t)((t + 1) / kPreStages) & 1u,
                                            c.err, dead);
                     tc_fence_after();
                     issue_s(a, t + 1);
+                    if (a == kPreQTiles - 1) umma_commit(bar(EMPTY_K + (t + 1) % kPreStages));
                 }
             }
         }
@@ -398,21 +433,39 @@ cascade_prefix_kernel(const __grid_constant__ CUtensorMap tmap, const __grid_con
         // ---- this CTA's record per (sharer, KV head) ----
         wait_phase(o_done(a), (uint32_t)(nt - 1) & 1u, c.err, dead);
         tc_fence_after();
-        float *rec = row_ok ? c.ws_pre + (((int64_t)ks * c.S + __ldcg(members + mrow)) * c.Hkv + g) * MF : nullptr;
+        float *rec = row_ok && !dead
+                         ? c.ws_pre + (((int64_t)ks * c.S + __ldcg(members + mrow)) * c.Hkv + g) * MF
+                         : nullptr;
         const int hl = r % G;
+        // O leaves through shared memory, 32 columns at a time, so that eight
+        // lanes write 128 consecutive bytes of a record (a lane writing its
+        // own row spread each store over 32 lines: the last step of a CTA,
+        // from the last P on, took 6 us).  The buffer is the stage that the
+        // last key tile did not use: every MMA that reads it was issued
+        // before the P.V just completed.
+        float *xb = reinterpret_cast<float *>(smem + L::ST_OFF + (nt % kPreStages) * L::STAGE) + warp * 32 * 32;
+        static_assert(SOFT_THREADS / 32 * 32 * 32 * 4 <= L::STAGE, "a 32 x 32 block per softmax warp");
+        const unsigned long long orow = rec ? reinterpret_cast<unsigned long long>(rec + hl * D) : 0ull;
         uint32_t v[32];
 #pragma unroll
         for (int cb = 0; cb < D / 32; ++cb) {
             tmem_ld32(trow + O_COL + cb * 32, v);
             tmem_wait_ld();
-            if (row_ok && !dead)
 #pragma unroll
-                for (int i = 0; i < 32; i += 4)
-                    *reinterpret_cast<float4 *>(rec + hl * D + cb * 32 + i) =
-                        make_float4(__uint_as_float(v[i]), __uint_as_float(v[i + 1]), __uint_as_float(v[i + 2]),
-                                    __uint_as_float(v[i + 3]));
+            for (int i = 0; i < 8; ++i)
+                *reinterpret_cast<uint4 *>(xb + lane * 32 + ((i ^ (lane & 7)) * 4)) =
+                    make_uint4(v[4 * i], v[4 * i + 1], v[4 * i + 2], v[4 * i + 3]);
+            __syncwarp();
+#pragma unroll
+            for (int i = 0; i < 8; ++i) {
+                const int rr = i * 4 + lane / 8, ch = lane % 8;  // row, 16-byte chunk
+                const unsigned long long dst = __shfl_sync(0xffffffffu, orow, rr);
+                const uint4 w = *reinterpret_cast<const uint4 *>(xb + rr * 32 + ((ch ^ (rr & 7)) * 4));
+                if (dst) *reinterpret_cast<uint4 *>(reinterpret_cast<float *>(dst) + cb * 32 + ch * 4) = w;
+            }
+            __syncwarp();
         }
-        if (row_ok && !dead) {
+        if (rec) {
             rec[G * D + hl] = m_run;
             rec[G * D + G + hl] = l_run;
         }
