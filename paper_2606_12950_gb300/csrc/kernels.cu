@@ -453,6 +453,12 @@ int kv_cascade_workspace_bytes(const kv_pool *p, int layout, int S, int Hq, int 
 
 namespace {
 
+// the model behind the choice of a prefix's key splits (attn_call)
+constexpr double kSuffixGuess = 512;         // tokens of a sequence after its prefix
+constexpr double kStreamBytesPerUs = 6.5e6;  // of the decode kernel
+constexpr double kSplitUs = 10;              // a prefix CTA's start and end
+constexpr double kKeyTileUs = 2.7;           // its 128-key tile, beside the decode kernel
+
 struct CascadePlan {
     const kv_prefix_group *groups;
     int n_groups;
@@ -604,10 +610,32 @@ int attn_call(kv_pool *p, int layout, const uint16_t *q, const uint16_t *k_new, 
     int P_pre = 0;
     rc = cascade_dispatch(L.head_dim, G, nullptr, c, 0, p->sm_count, nullptr, false, &P_pre);
     if (rc) return rc;
-    // key splits: as many as keep the prefix grid within a quarter of the
-    // GPU's CTA slots for it (at least one; every split non-empty)
-    const int pre_slots = std::max(1, P_pre / 4);
-    c->KS = std::max(1, std::min({pre_slots / std::max(1, tiles * Hkv), kvp::kMaxKeySplits, kt_min}));
+    // Key splits: as many as keep the prefix grid within a quarter of the
+    // GPU's CTA slots for it (at least one; every split non-empty).  If a split
+    // would still take longer than the suffixes beside it, more, up to 3/7 of
+    // the slots (64 SMs).  The lengths are on the device, so the suffixes are
+    // taken for kSuffixGuess tokens each.  A split takes about kSplitUs plus
+    // kKeyTileUs per 128 keys.  Measured, one step in us, at the quarter's
+    // rule and at this one (splits): 190 suffixes of about 500 tokens, 3
+    // groups, 4096-token prefixes 115 (1) and 84 (2); 200 of about 500, one
+    // 8192-token prefix 192 (1) and 95 (2); 128 of about 100, 2 groups, 4096
+    // tokens 57 (2) and 46 (3); 12 of about 500, 4096 tokens 30 (4) and 21 (8);
+    // 120 of about 2900, 3 groups, 4096 tokens 261 (1) and 259 (2).  Where the
+    // suffixes are much longer than the guess it can cost them a little: 361
+    // of about 3900, 4 groups, 3968 tokens, one KV head at d = 64, 69.7 (4)
+    // and 71.8 (8).  Past 3/7 the suffixes lose more than the prefix gains
+    // (8192 tokens: 113 with 4 splits on 128 SMs), and so they do where the
+    // prefix is no longer than they are (256 of about 500 tokens, 2048-token
+    // prefix: 101 with 1 split, 108 with 2).
+    const int pre_base = std::max(1, tiles * Hkv);
+    const int ks_most = std::min(kvp::kMaxKeySplits, kt_min);
+    c->KS = std::max(1, std::min(P_pre / 4 / pre_base, ks_most));
+    int kt_max = 0;
+    for (int i = 0; i < ng; ++i) kt_max = std::max(kt_max, tokens[i] / kvp::kPreChunk);
+    const double suffix_us = (double)S * kSuffixGuess * (4.0 * Hkv * L.head_dim) / kStreamBytesPerUs;
+    while (c->KS < ks_most && pre_base * (c->KS + 1) <= P_pre * 3 / 7 &&
+           kSplitUs + kKeyTileUs * (kt_max / 2.0) / c->KS > suffix_us)
+        ++c->KS;
     // the decode grid fills the SMs the prefix grid leaves free (all of them
     // when the prefix grid needs more than half the GPU: the decode CTAs then
     // start as prefix CTAs finish)

@@ -153,3 +153,27 @@ def test_cta_level_parts_with_a_shared_prefix():
     assert np.array_equal(pool.download(), ref_pool)
     _check(db.out_f64(), oracle.batch_attention(b, pool=ref_pool), "prefix")
     assert pool.error() == 0
+
+
+@pytest.mark.parametrize("G,Hkv,d", [(4, 8, 128), (8, 1, 128), (2, 2, 64)])
+@pytest.mark.parametrize("tokens", [64, 192, 448, 576, 4160])
+def test_key_splits_of_a_shared_prefix(tokens, G, Hkv, d):
+    """Few members, so the prefix is cut into as many key splits as it has
+    64-token chunks, eight at most: splits of one chunk (a half tile), of an
+    odd number of chunks, and of more tiles than are asked of L2 ahead."""
+    from paper_2606_12950_gb300 import kvpool as K
+    from paper_2606_12950_gb300.runner import DeviceBatch, DevicePool
+
+    groups = [([0, 1, 2], tokens), ([4, 5], tokens)]
+    pre = [tokens, tokens + 16, tokens + 333, 50, tokens, tokens + 100]
+    b = W.make_batch(7400 + tokens + G, pre, Hq=G * Hkv, Hkv=Hkv, d=d, bs=16, extra_blocks=3)
+    W.share_prefix(b, groups)
+    pool = DevicePool(b.n_pages, b.page_elems * 2, b.bs, [(b.Hkv, b.d)])
+    pool.upload(b.pool)
+    db = DeviceBatch(pool, 0, b)
+    db.cascade(K.PrefixPlan(groups))
+    torch.cuda.synchronize()
+    ref_pool = oracle.batch_append(b)
+    assert np.array_equal(pool.download(), ref_pool)
+    _check(db.out_f64(), oracle.batch_attention(b, pool=ref_pool), (tokens, G))
+    assert pool.error() == 0
