@@ -25,7 +25,7 @@
 // one mbarrier for K and one for V: the next unit's K streams in while the
 // warp does softmax and P.V on the current one, the next V while it does the
 // next q.K.  (Measured on GB300: one issuing thread per SM cannot keep HBM
-// busy with these 2 KB boxes; one per warp can.)  The pool rows of the CTA's
+// busy with these 2 KB boxes; one per warp can.)  The pool rows of a warp's
 // units are resolved from the block table in the prologue, while the memory
 // system is idle, so no table load sits on the streaming path, and each
 // run's q rows (and, for the run's last tile, this step's new K/V rows) are
@@ -142,6 +142,7 @@ struct AttnArgs {
     int32_t S;
     int32_t Hkv;
     int32_t bs;
+    int32_t bs_shift;        // log2(bs), or -1
     int32_t rows_cap;        // boxes whose pool rows are resolved up front
     int32_t P;               // CTAs
     int32_t nwarps;          // warps per CTA (<= kWarps), one part each
@@ -592,12 +593,35 @@ struct MmaCompute {
 };
 
 // ----------------------------------------------------------- work units ---
-struct Piece {
-    int32_t pb, pe;        // piece unit range
-    int32_t run_begin;     // unit id of tile 0 of this (s, g) run
-    int32_t run_end;
-    int32_t s, g, n;       // sequence, KV head, context length
-    int32_t skip;          // leading tokens handled by the prefix kernel
+// Index arithmetic.  It is on the critical path of every step (lengths, parts,
+// table rows: 4.4 us from a grid's start to its first loads, of which two
+// round trips to L2 are 1.2) and again at each run boundary.  So parts take
+// 32-bit arithmetic with one division, quotients below 2^20 an estimate from
+// the approximate reciprocal, a warp looks up its own rows without a CTA
+// barrier, and the run after a piece is stepped to instead of searched for.
+// Against 64-bit divisions, a CTA-wide lookup and a search per piece (same
+// box): the 64-sequence layer (435 MB) 70.1 -> 67.8 us, 256 chains beside
+// their prefix 100.7 -> 95.5, 128 sequences at d = 64 74.0 -> 69.8, three
+// co-located models 281.7 -> 277.5, 1024 long contexts 705.7 -> 699.0.
+//
+// x / d for a quotient below 2^20 (x and d positive and below 2^31), inv =
+// 1 / d to within 2 ulp: three roundings of 2^-23 at most make the estimate
+// less than one off, so its floor is off by one at most.
+__device__ __forceinline__ int32_t div_est(uint32_t x, uint32_t d, float inv)
+{
+    int32_t q = (int32_t)((float)x * inv);
+    const int32_t r = (int32_t)(x - (uint32_t)q * d);
+    if (r < 0) --q;
+    if (r >= (int32_t)d) ++q;
+    return q;
+}
+__device__ __forceinline__ float inv_of(int32_t d) { return __fdividef(1.f, (float)d); }
+
+// A run: the units of one (sequence, KV head).
+struct Run {
+    int32_t s, g;   // sequence, KV head
+    int32_t nt;     // units
+    int32_t begin;  // id of the first one
 };
 
 // Context length of sequence s, read once per CTA in the prologue and clamped
@@ -648,19 +672,39 @@ __device__ __forceinline__ int find_seq(const int32_t *T, int S, int32_t u)
     return lo;
 }
 
-__device__ __forceinline__ void decode_piece(const AttnArgs &a, const int32_t *T, int32_t u, int32_t u1, Piece &p)
+// units of a run of sequence s
+template <int D>
+__device__ __forceinline__ int32_t run_units(const int32_t *T, int S, int s)
 {
-    const int s = find_seq(T, a.S, u);
-    const int32_t nt = (T[s + 1] - T[s]) / a.Hkv;
-    const int32_t g = (u - T[s]) / nt;
-    p.s = s;
-    p.g = g;
-    p.n = seq_len(T, a.S, s);
-    p.skip = seq_skip(T, a.S, s);
-    p.run_begin = T[s] + g * nt;
-    p.run_end = p.run_begin + nt;
-    p.pb = u;
-    p.pe = p.run_end < u1 ? p.run_end : u1;
+    return (int32_t)((uint32_t)(seq_len(T, S, s) - seq_skip(T, S, s) + kUnit<D> - 1) / (uint32_t)kUnit<D>);
+}
+
+// the run that holds unit u
+template <int D>
+__device__ __forceinline__ Run run_of(const AttnArgs &a, const int32_t *T, int32_t u)
+{
+    Run r;
+    r.s = find_seq(T, a.S, u);
+    r.nt = run_units<D>(T, a.S, r.s);
+    const int32_t t0 = T[r.s];
+    r.g = div_est((uint32_t)(u - t0), (uint32_t)r.nt, inv_of(r.nt));
+    r.begin = t0 + r.g * r.nt;
+    return r;
+}
+
+// the run after r (there is one: the caller has units past r)
+template <int D>
+__device__ __forceinline__ Run next_run(const AttnArgs &a, const int32_t *T, Run r)
+{
+    r.begin += r.nt;
+    if (++r.g == a.Hkv) {
+        r.g = 0;
+        do
+            ++r.s;
+        while (T[r.s + 1] == T[r.s]);  // sequences without units
+        r.nt = run_units<D>(T, a.S, r.s);
+    }
+    return r;
 }
 
 // Block table entry idx (flat): this step's value when the table sync is
@@ -682,19 +726,17 @@ constexpr int32_t kRowBad = -1, kRowNone = -2;
 template <int D>
 __device__ __forceinline__ int32_t unit_row(const AttnArgs &a, const int32_t *T, int32_t u, int j)
 {
-    const int s = find_seq(T, a.S, u);
-    const int32_t nt = (T[s + 1] - T[s]) / a.Hkv;
-    const int32_t within = u - T[s];
-    const int32_t g = within / nt;
-    const int32_t tok0 = seq_skip(T, a.S, s) + (within - g * nt) * kUnit<D> + j * kTile;
-    if (j > 0 && tok0 >= seq_len(T, a.S, s)) return kRowNone;
-    const int32_t phys = table_entry(a, (int64_t)s * a.max_blocks + tok0 / a.bs);
+    const Run r = run_of<D>(a, T, u);
+    const int32_t tok0 = seq_skip(T, a.S, r.s) + (u - r.begin) * kUnit<D> + j * kTile;
+    if (j > 0 && tok0 >= seq_len(T, a.S, r.s)) return kRowNone;
+    const int32_t blk = a.bs_shift >= 0 ? tok0 >> a.bs_shift : tok0 / a.bs;
+    const int32_t phys = table_entry(a, (int64_t)r.s * a.max_blocks + blk);
     if (phys < 0 || (int64_t)phys + a.pages_per_block > a.pool_pages) return kRowBad;
-    return (int32_t)((int64_t)phys * a.rows_per_page + (tok0 % a.bs) + (int64_t)g * a.bs);
+    return (int32_t)((int64_t)phys * a.rows_per_page + (tok0 - blk * a.bs) + (int64_t)r.g * a.bs);
 }
 
 // the part (of NP) whose range contains unit u
-__device__ __forceinline__ int32_t cta_of(int64_t u, int64_t W, int64_t P)
+__device__ __forceinline__ int32_t part_of(int64_t u, int64_t W, int64_t P)
 {
     return (int32_t)(((u + 1) * P - 1) / W);
 }
@@ -869,18 +911,20 @@ paged_attn_kernel(const __grid_constant__ CUtensorMap tmap, const __grid_constan
         }
         if (lane == 31) misc[warp] = incl;
         __syncthreads();
-        int32_t base = 0;
-        for (int w = 0; w < warp; ++w) base += misc[w];
-        int32_t run = base + incl - local;
+        int32_t sums = lane < NW ? misc[lane] : 0;  // of the warps up to this lane's
+#pragma unroll
+        for (int off = 1; off < kWarps; off <<= 1) {
+            const int32_t v = __shfl_up_sync(0xffffffffu, sums, off);
+            if (lane >= off) sums += v;
+        }
+        const int32_t base = __shfl_sync(0xffffffffu, sums, warp > 0 ? warp - 1 : 0);
+        const int32_t tot = __shfl_sync(0xffffffffu, sums, kWarps - 1);
+        int32_t run = (warp > 0 ? base : 0) + incl - local;
         for (int s = lo; s < hi; ++s) {  // this thread's own NL / SK entries
             T[s] = run;
-            run += ((seq_len(T, S, s) - seq_skip(T, S, s) + UNIT - 1) / UNIT) * Hkv;
+            run += run_units<D>(T, S, s) * Hkv;
         }
-        if (tid == 0) {
-            int32_t tot = 0;
-            for (int w = 0; w < NW; ++w) tot += misc[w];
-            T[S] = tot;
-        }
+        if (tid == 0) T[S] = tot;
         if (early) {
             if (a.chain == 0) grid_dependency_wait();
             write_sync();
@@ -908,38 +952,38 @@ paged_attn_kernel(const __grid_constant__ CUtensorMap tmap, const __grid_constan
     // exactly the parts part_of(first unit) .. part_of(last unit).  A part
     // gets at least MIN_UNITS units when the batch is small (fewer
     // partials to write and merge; enough warps still stream to fill HBM).
-    const int64_t W = T[S];
+    const int32_t W = T[S];
     constexpr int MIN_UNITS = kMinPartTokens / UNIT;
-    const int64_t most = MERGE ? (int64_t)a.P : (int64_t)a.P * NW;
-    const int64_t fine = MERGE ? (W + NW - 1) / NW : W / MIN_UNITS > 0 ? W / MIN_UNITS : W;
-    const int64_t NP = fine < most ? fine : most;
-    const int64_t first_part = MERGE ? (int64_t)blockIdx.x : (int64_t)blockIdx.x * NW;
-    if (first_part >= NP) {
+    const int32_t most = MERGE ? a.P : a.P * NW;
+    const int32_t fine = MERGE ? (W + NW - 1) / NW : W / MIN_UNITS > 0 ? W / MIN_UNITS : W;
+    const int32_t NP = fine < most ? fine : most;
+    const int32_t first_part = MERGE ? (int32_t)blockIdx.x : (int32_t)blockIdx.x * NW;
+    const int32_t part = MERGE ? first_part : first_part + warp;
+    if ((MERGE ? first_part : part) >= NP) {  // no CTA-wide barrier below this point without MERGE
         if (chained) grid_dependency_wait();
         return;
     }
-    const int64_t last_part = MERGE ? first_part + 1 : first_part + NW < NP ? first_part + NW : NP;  // exclusive
-    const int32_t cu0 = (int32_t)(first_part * W / NP);                             // this CTA's units
-    const int32_t cu1 = (int32_t)(last_part * W / NP);
+    // first unit of part p: p * W / NP, with W = wq * NP + wr
+    const int32_t wq = (int32_t)((uint32_t)W / (uint32_t)NP), wr = W - wq * NP;
+    const float np_inv = inv_of(NP);
+    auto part_begin = [&](int32_t p) {
+        return NP < 65536 / 2 ? p * wq + div_est((uint32_t)p * (uint32_t)wr, (uint32_t)NP, np_inv)
+                              : (int32_t)((int64_t)p * W / NP);
+    };
+    const int32_t g0 = part_begin(part), g1 = part_begin(part + 1);  // this part's units
+    const int32_t cu0 = MERGE ? g0 : part_begin(first_part);         // this CTA's first
+    const int32_t nu = g1 - g0;
+    // this warp's units: the part's without MERGE
+    const int32_t u0 = MERGE ? g0 + warp * nu / NW : g0;
+    const int32_t u1 = MERGE ? g0 + (warp + 1) * nu / NW : g1;
 
-    // ---- prologue 2: resolve the block table for this CTA's units while the
+    // ---- prologue 2: resolve the block table for this warp's units while the
     // memory system is idle (later lookups would queue behind the TMA stream)
     {
-        const int32_t nr = min((cu1 - cu0) * SUB, a.rows_cap);
-        for (int32_t k = tid; k < nr; k += NT) rows[k] = unit_row<D>(a, T, cu0 + k / SUB, k % SUB);
-        __syncthreads();
+        const int32_t k0 = (u0 - cu0) * SUB, k1 = min((u1 - cu0) * SUB, a.rows_cap);
+        for (int32_t k = k0 + lane; k < k1; k += 32) rows[k] = unit_row<D>(a, T, cu0 + k / SUB, k % SUB);
+        __syncwarp();
     }
-
-    const int64_t part = MERGE ? first_part : first_part + warp;
-    if (part >= NP) {  // no CTA-wide barrier below this point without MERGE
-        if (chained) grid_dependency_wait();
-        return;
-    }
-    // this warp's units [u0, u1), and its part's [g0, g1): the same without MERGE
-    const int32_t nu = cu1 - cu0;
-    const int32_t u0 = MERGE ? cu0 + warp * nu / NW : (int32_t)(part * W / NP);
-    const int32_t u1 = MERGE ? cu0 + (warp + 1) * nu / NW : (int32_t)((part + 1) * W / NP);
-    const int32_t g0 = MERGE ? cu0 : u0, g1 = MERGE ? cu1 : u1;
     float *mbuf = reinterpret_cast<float *>(mbufs) + (size_t)warp * MF;
     if (MERGE && lane == 0) {
         chains[warp].x = -1;
@@ -966,11 +1010,14 @@ paged_attn_kernel(const __grid_constant__ CUtensorMap tmap, const __grid_constan
     uint8_t *qb = qbufs + (size_t)warp * QB;
     uint8_t *ab = abufs + (size_t)warp * AB;
     const uint32_t qb_addr = smem_u32(qb), ab_addr = smem_u32(ab);
-    {
-        const int s0 = find_seq(T, S, MERGE && u0 == u1 ? cu0 : u0);
-        const int32_t nt0 = (T[s0 + 1] - T[s0]) / Hkv;
-        const uint16_t *src = a.q + ((int64_t)s0 * Hq + (int64_t)(((MERGE && u0 == u1 ? cu0 : u0) - T[s0]) / nt0) * G) * D;
+    auto stage_q = [&](const Run &r) {
+        const uint16_t *src = a.q + ((int64_t)r.s * Hq + (int64_t)r.g * G) * D;
         for (uint32_t c = lane; c < QB / 16; c += 32) cp_async16(qb_addr + c * 16, src + c * 8);
+    };
+    Run run{};
+    if (!MERGE || u0 < u1) {
+        run = run_of<D>(a, T, u0);
+        stage_q(run);
         cp_async_commit();
     }
 
@@ -978,8 +1025,8 @@ paged_attn_kernel(const __grid_constant__ CUtensorMap tmap, const __grid_constan
     uint32_t consumed = 0;
     int32_t u = u0;
     while (u < u1) {
-        Piece pc;
-        decode_piece(a, T, u, u1, pc);
+        const int32_t n = seq_len(T, S, run.s), skip = seq_skip(T, S, run.s);
+        const int32_t run_end = run.begin + run.nt, pe = run_end < u1 ? run_end : u1;  // the piece: [u, pe)
         cp_async_wait_all();  // this piece's q rows
         __syncwarp();
         Comp comp;
@@ -987,28 +1034,27 @@ paged_attn_kernel(const __grid_constant__ CUtensorMap tmap, const __grid_constan
         __syncwarp();  // every lane holds its q fragments: the buffer may be refilled
         // fused append: the run's last tile holds position n-1, whose K/V row
         // is this step's new token; this warp alone reads that tile
-        const bool app_run = a.k_new != nullptr && pc.pe == pc.run_end && !seq_len_clamped(T, S, pc.s);
+        const bool app_run = a.k_new != nullptr && pe == run_end && !seq_len_clamped(T, S, run.s);
         if (app_run && lane < AB / 16) {
             const int which = lane / (D / 8), c = lane % (D / 8);
-            cp_async16(ab_addr + lane * 16, (which ? a.v_new : a.k_new) + ((int64_t)pc.s * Hkv + pc.g) * D + c * 8);
+            cp_async16(ab_addr + lane * 16, (which ? a.v_new : a.k_new) + ((int64_t)run.s * Hkv + run.g) * D + c * 8);
         }
-        if (pc.pe < u1) {  // the next piece's q rows
-            const int s2 = find_seq(T, S, pc.pe);
-            const int32_t nt2 = (T[s2 + 1] - T[s2]) / Hkv;
-            const uint16_t *src = a.q + ((int64_t)s2 * Hq + (int64_t)((pc.pe - T[s2]) / nt2) * G) * D;
-            for (uint32_t c = lane; c < QB / 16; c += 32) cp_async16(qb_addr + c * 16, src + c * 8);
+        Run next = run;
+        if (pe < u1) {  // the next piece's q rows
+            next = next_run<D>(a, T, run);
+            stage_q(next);
         }
         cp_async_commit();
-        for (int32_t uu = pc.pb; uu < pc.pe; ++uu) {
+        for (int32_t uu = u; uu < pe; ++uu) {
             const int st = (int)(consumed % kStages);
             const uint32_t par = (consumed / kStages) & 1u;
             uint8_t *Ks = k_of(st);
             uint8_t *Vs = Ks + TILE_BYTES;
             const uint32_t bk = bk_of(st), bv = bv_of(st);
-            const int nvalid = min(UNIT, pc.n - pc.skip - (uu - pc.run_begin) * UNIT);
+            const int nvalid = min(UNIT, n - skip - (uu - run.begin) * UNIT);
             const bool more = uu + kStages < u1;  // the unit this stage takes next
-            const bool app = app_run && uu == pc.run_end - 1;
-            const int arow = (pc.n - 1 - pc.skip) % UNIT;
+            const bool app = app_run && uu == run_end - 1;
+            const int arow = (n - 1 - skip) % UNIT;
             wait_phase(bk, par, a.err, dead);
             if (app) {
                 cp_async_wait_all();  // the new K/V rows
@@ -1051,29 +1097,30 @@ paged_attn_kernel(const __grid_constant__ CUtensorMap tmap, const __grid_constan
         }
 
         // ---- end of a piece: the output, or this part's partial ----
-        const int32_t r = pc.s * Hkv + pc.g;
-        const int32_t p_first = cta_of(pc.run_begin, W, NP);
-        const int32_t p_last = cta_of(pc.run_end - 1, W, NP);
+        const int32_t r = run.s * Hkv + run.g;
         // a run whose prefix lives in prefix records always leaves a partial
-        const bool split = p_first != p_last || pc.skip > 0;
-        uint16_t *orow = a.out + ((int64_t)pc.s * Hq + (int64_t)pc.g * G) * D;
+        const bool split = run.begin < g0 || run_end > g1 || skip > 0;
+        // parts of the run that starts in this one (told to the combine)
+        auto parts = [&]() { return !split ? 0 : run_end > g1 ? part_of(run_end - 1, W, NP) - part + 1 : 1; };
+        uint16_t *orow = a.out + ((int64_t)run.s * Hq + (int64_t)run.g * G) * D;
         float *slot = a.ws_part + ((int64_t)r + part) * MF;
         // (MERGE) the part's share of the run; it may go on over several warps
-        const int32_t lo = pc.run_begin > g0 ? pc.run_begin : g0, hi = pc.run_end < g1 ? pc.run_end : g1;
-        if (!MERGE || (pc.pb == lo && pc.pe == hi)) {
+        const int32_t lo = run.begin > g0 ? run.begin : g0, hi = run_end < g1 ? run_end : g1;
+        if (!MERGE || (u == lo && pe == hi)) {
             make_ready();
             comp.store(orow, slot, split, lane);
-            if (part == p_first && lane == 0)  // each run has one first part: it tells the combine
-                a.ws_run[r] = make_int2(p_first, split ? p_last - p_first + 1 : 0);
-        } else if (pc.pb != lo) {  // goes on from an earlier warp, whose chain merges it
+            if (run.begin >= g0 && lane == 0)  // each run has one first part: it tells the combine
+                a.ws_run[r] = make_int2(part, parts());
+        } else if (u != lo) {  // goes on from an earlier warp, whose chain merges it
             comp.store(nullptr, mbuf, true, lane);
         } else {  // goes on in the next warp: the last piece here, so the stage is free
             comp.store(nullptr, reinterpret_cast<float *>(wstage), true, lane);
             if (lane == 0)
-                chains[warp] = make_int4(r, (int)(((int64_t)(hi - cu0) * NW - 1) / nu) - warp, p_first,
-                                         split ? p_last - p_first + 1 : 0);
+                chains[warp] = make_int4(r, ((hi - g0) * NW - 1) / nu - warp, run.begin >= g0 ? 1 : 0,
+                                         run.begin >= g0 || !split ? parts() : 1);
         }
-        u = pc.pe;
+        u = pe;
+        run = next;
     }
     if constexpr (MERGE) {
         __syncthreads();
@@ -1104,7 +1151,7 @@ paged_attn_kernel(const __grid_constant__ CUtensorMap tmap, const __grid_constan
                     slot[G * D + G + h] = L;
                 }
             }
-            if (c == 0 && ch.z == (int)part) a.ws_run[ch.x] = make_int2(ch.z, ch.w);
+            if (c == 0 && ch.z) a.ws_run[ch.x] = make_int2(part, ch.w);
         }
     }
     if (chained) grid_dependency_wait();

@@ -86,6 +86,9 @@ int attn_run(const CUtensorMap *tmap, AttnArgs a, int P_req, int sm_count, cudaS
     *P_out = P;
     if (what == kLaunchQuery) return KV_OK;
     a.rows_cap = kRowsCap;
+    a.bs_shift = -1;
+    for (int k = 4; k < 31; ++k)
+        if (a.bs == 1 << k) a.bs_shift = k;
     a.P = P;
     // A batch whose table has room for fewer than kMergeUnits units a warp
     // runs with its CTAs as the parts (MERGE), if the merge's buffers cost no
