@@ -271,7 +271,7 @@ struct FmaCompute {
     }
 
     // q.K for the tile's tokens, online-softmax update, weights p
-    __device__ __forceinline__ void qk(const uint8_t *Ks, int nvalid)
+    __device__ __forceinline__ void scores(const uint8_t *Ks, int nvalid)
     {
         nv = nvalid;
         float sc[TPG][G];
@@ -338,6 +338,8 @@ struct FmaCompute {
                 l[h] += p[i][h];
             }
     }
+
+    __device__ __forceinline__ void softmax() {}
 
     // o += p * V for the tile's valid tokens
     __device__ __forceinline__ void pv(uint8_t *Vs)
@@ -419,6 +421,7 @@ struct MmaCompute {
     uint32_t qf[KS][2];  // B operand of q.K: Q^T fragments (bf16x2)
     float acc[KS][4];    // O^T accumulators, 16 d-rows per block
     float m[2], l[2];    // heads 2*tig, 2*tig+1
+    float x[NM][4];      // scores of the unit
     uint32_t pb[NM][2];  // B operand of P.V (P^T fragments)
     float qk_scale;
     int gid, tig, lane_, nv;
@@ -446,15 +449,13 @@ struct MmaCompute {
         l[0] = l[1] = 0.f;
     }
 
-    __device__ __forceinline__ void qk(const uint8_t *Ks, int nvalid)
+    // q.K.  (Two sums of every other 16 columns, a chain of MMAs half as long,
+    // left the 64-sequence layer at 68.2 us against 67.8 with one.)
+    __device__ __forceinline__ void scores(const uint8_t *Ks, int nvalid)
     {
         nv = nvalid;
         const uint32_t kbase = smem_u32(Ks);
         const int mat = lane_ >> 3, r8 = lane_ & 7;
-        // rows past the valid tokens of a loaded box may hold anything; a box
-        // that was not loaded (16 mt >= nvalid) holds an earlier
-        // unit's rows: both are masked
-        float x[NM][4];
 #pragma unroll
         for (int mt = 0; mt < NM; ++mt) {
             float s[4] = {0.f, 0.f, 0.f, 0.f};
@@ -464,12 +465,24 @@ struct MmaCompute {
                 ldmatrix_x4(kbase + swz(mt * 16 + r8 + (mat & 1) * 8, kk * 2 + (mat >> 1)), a0, a1, a2, a3);
                 mma_bf16_16816(s, a0, a1, a2, a3, qf[kk][0], qf[kk][1]);
             }
-            // s[0], s[1]: token gid, heads 2tig, 2tig+1; s[2], s[3]: token gid+8
-            const bool ok0 = mt * 16 + gid < nvalid, ok1 = mt * 16 + gid + 8 < nvalid;
-            x[mt][0] = ok0 ? s[0] * qk_scale : -INFINITY;
-            x[mt][1] = ok0 ? s[1] * qk_scale : -INFINITY;
-            x[mt][2] = ok1 ? s[2] * qk_scale : -INFINITY;
-            x[mt][3] = ok1 ? s[3] * qk_scale : -INFINITY;
+#pragma unroll
+            for (int e = 0; e < 4; ++e) x[mt][e] = s[e] * qk_scale;
+        }
+    }
+
+    // online softmax of the scores: the weights P as P.V's operand
+    __device__ __forceinline__ void softmax()
+    {
+        // x[0], x[1]: token gid, heads 2tig, 2tig+1; x[2], x[3]: token gid+8.
+        // Rows past the valid tokens of a loaded box may hold anything; a box
+        // that was not loaded (16 mt >= nv) holds an earlier unit's rows: both
+        // are masked
+        if (nv < kUnit<D>) {
+#pragma unroll
+            for (int mt = 0; mt < NM; ++mt) {
+                if (mt * 16 + gid >= nv) x[mt][0] = x[mt][1] = -INFINITY;
+                if (mt * 16 + gid + 8 >= nv) x[mt][2] = x[mt][3] = -INFINITY;
+            }
         }
         float t0 = fmaxf(x[0][0], x[0][2]), t1 = fmaxf(x[0][1], x[0][3]);
 #pragma unroll
@@ -477,31 +490,34 @@ struct MmaCompute {
             t0 = fmaxf(t0, fmaxf(x[mt][0], x[mt][2]));
             t1 = fmaxf(t1, fmaxf(x[mt][1], x[mt][3]));
         }
+        // lazy rescale (see FmaCompute::scores); the maxima over the tokens are
+        // only needed once some lane's exceeds the running one by 2^8
+        if (__any_sync(0xffffffffu, t0 > m[0] + 8.f || t1 > m[1] + 8.f)) {
 #pragma unroll
-        for (int off = 4; off < 32; off <<= 1) {
-            t0 = fmaxf(t0, __shfl_xor_sync(0xffffffffu, t0, off));
-            t1 = fmaxf(t1, __shfl_xor_sync(0xffffffffu, t1, off));
-        }
-        // lazy rescale (see FmaCompute::qk)
-        if (t0 > m[0] + 8.f) {
-            const float a = fast_exp2(m[0] - t0);
-            l[0] *= a;
-#pragma unroll
-            for (int mb = 0; mb < KS; ++mb) {
-                acc[mb][0] *= a;
-                acc[mb][2] *= a;
+            for (int off = 4; off < 32; off <<= 1) {
+                t0 = fmaxf(t0, __shfl_xor_sync(0xffffffffu, t0, off));
+                t1 = fmaxf(t1, __shfl_xor_sync(0xffffffffu, t1, off));
             }
-            m[0] = t0;
-        }
-        if (t1 > m[1] + 8.f) {
-            const float a = fast_exp2(m[1] - t1);
-            l[1] *= a;
+            if (t0 > m[0] + 8.f) {
+                const float a = fast_exp2(m[0] - t0);
+                l[0] *= a;
 #pragma unroll
-            for (int mb = 0; mb < KS; ++mb) {
-                acc[mb][1] *= a;
-                acc[mb][3] *= a;
+                for (int mb = 0; mb < KS; ++mb) {
+                    acc[mb][0] *= a;
+                    acc[mb][2] *= a;
+                }
+                m[0] = t0;
             }
-            m[1] = t1;
+            if (t1 > m[1] + 8.f) {
+                const float a = fast_exp2(m[1] - t1);
+                l[1] *= a;
+#pragma unroll
+                for (int mb = 0; mb < KS; ++mb) {
+                    acc[mb][1] *= a;
+                    acc[mb][3] *= a;
+                }
+                m[1] = t1;
+            }
         }
 #pragma unroll
         for (int mt = 0; mt < NM; ++mt) {
@@ -770,23 +786,35 @@ __device__ __forceinline__ void store_column(uint16_t *dst, const float4 &O, flo
     *reinterpret_cast<uint2 *>(dst) = make_uint2(*reinterpret_cast<uint32_t *>(&lo), *reinterpret_cast<uint32_t *>(&hi));
 }
 
-// Load K (which = 0) or V (which = 1) of unit u into this warp's stage;
+// The pool rows of a unit's boxes (lane 0's).
+template <int D>
+struct UnitRows {
+    int32_t y[kSub<D>];
+};
+template <int D>
+__device__ __forceinline__ UnitRows<D> rows_of(const AttnArgs &a, const int32_t *T, const int32_t *rows, int32_t cu0,
+                                               int32_t u)
+{
+    UnitRows<D> r;
+    const int32_t k = (u - cu0) * kSub<D>;
+#pragma unroll
+    for (int j = 0; j < kSub<D>; ++j) r.y[j] = k + j < a.rows_cap ? rows[k + j] : unit_row<D>(a, T, u, j);
+    return r;
+}
+
+// Load K (which = 0) or V (which = 1) of a unit into this warp's stage;
 // completes on `bar`.  Lane 0 only.
 template <int D>
-__device__ __forceinline__ void issue_half(const CUtensorMap *tmap, const AttnArgs &a, const int32_t *T,
-                                           const int32_t *rows, int32_t cu0, int32_t u, int which, uint32_t dst,
-                                           uint32_t bar, uint64_t policy)
+__device__ __forceinline__ void issue_half(const CUtensorMap *tmap, const AttnArgs &a, const UnitRows<D> &r, int which,
+                                           uint32_t dst, uint32_t bar, uint64_t policy)
 {
     constexpr int HALVES = D / 64, SUB = kSub<D>;
-    const int32_t k = (u - cu0) * SUB;
-    int32_t y[SUB];
     uint32_t boxes = 0;
     bool bad = false;
 #pragma unroll
     for (int j = 0; j < SUB; ++j) {
-        y[j] = k + j < a.rows_cap ? rows[k + j] : unit_row<D>(a, T, u, j);
-        bad |= y[j] == kRowBad;
-        boxes += y[j] >= 0 ? 1u : 0u;
+        bad |= r.y[j] == kRowBad;
+        boxes += r.y[j] >= 0 ? 1u : 0u;
     }
     if (bad) {
         report(a.err, KV_ERR_DEVICE_BOUNDS);
@@ -796,10 +824,10 @@ __device__ __forceinline__ void issue_half(const CUtensorMap *tmap, const AttnAr
     mbar_arrive_expect_tx(bar, boxes * HALVES * kHalfBytes);
 #pragma unroll
     for (int j = 0; j < SUB; ++j)
-        if (SUB == 1 || y[j] >= 0)
+        if (SUB == 1 || r.y[j] >= 0)
 #pragma unroll
             for (int h = 0; h < HALVES; ++h)  // box (j, h): with SUB > 1, HALVES is 1
-                tma_load_2d(dst + (j + h) * kHalfBytes, tmap, h * 64, y[j] + which * a.Hkv * a.bs, bar, policy);
+                tma_load_2d(dst + (j + h) * kHalfBytes, tmap, h * 64, r.y[j] + which * a.Hkv * a.bs, bar, policy);
 }
 
 template <int D, int G, class Comp, bool MERGE>
@@ -1000,8 +1028,9 @@ paged_attn_kernel(const __grid_constant__ CUtensorMap tmap, const __grid_constan
 
     if (lane == 0) {
         for (int st = 0; st < kStages && u0 + st < u1; ++st) {
-            issue_half<D>(&tmap, a, T, rows, cu0, u0 + st, 0, smem_u32(k_of(st)), bk_of(st), policy);
-            issue_half<D>(&tmap, a, T, rows, cu0, u0 + st, 1, smem_u32(k_of(st) + TILE_BYTES), bv_of(st), policy);
+            const UnitRows<D> ur = rows_of<D>(a, T, rows, cu0, u0 + st);
+            issue_half<D>(&tmap, a, ur, 0, smem_u32(k_of(st)), bk_of(st), policy);
+            issue_half<D>(&tmap, a, ur, 1, smem_u32(k_of(st) + TILE_BYTES), bv_of(st), policy);
         }
     }
     // A run's q rows and, for the run's last tile, its new K/V rows are staged
@@ -1055,6 +1084,8 @@ paged_attn_kernel(const __grid_constant__ CUtensorMap tmap, const __grid_constan
             const bool more = uu + kStages < u1;  // the unit this stage takes next
             const bool app = app_run && uu == run_end - 1;
             const int arow = (n - 1 - skip) % UNIT;
+            UnitRows<D> ur;
+            if (more && lane == 0) ur = rows_of<D>(a, T, rows, cu0, uu + kStages);
             wait_phase(bk, par, a.err, dead);
             if (app) {
                 cp_async_wait_all();  // the new K/V rows
@@ -1063,12 +1094,16 @@ paged_attn_kernel(const __grid_constant__ CUtensorMap tmap, const __grid_constan
                     *reinterpret_cast<uint4 *>(Ks + swz(arow, lane)) = *reinterpret_cast<const uint4 *>(ab + lane * 16);
                 __syncwarp();
             }
-            comp.qk(Ks, nvalid);
-            // the K stage is refilled by TMA next: order the warp's generic
+            comp.scores(Ks, nvalid);
+            // K is asked for again as soon as its scores are done, before the
+            // softmax, from rows read before the wait: 1024 long contexts 704.3
+            // -> 702.5 us, one long sequence 14.7 -> 14.3.  The K stage is
+            // refilled by TMA next: order the warp's generic
             // shared-memory reads before the async-proxy write
             fence_proxy_async_smem();
             __syncwarp();
-            if (more && lane == 0) issue_half<D>(&tmap, a, T, rows, cu0, uu + kStages, 0, smem_u32(Ks), bk, policy);
+            if (more && lane == 0) issue_half<D>(&tmap, a, ur, 0, smem_u32(Ks), bk, policy);
+            comp.softmax();
             wait_phase(bv, par, a.err, dead);
             if (app) {
                 if (lane < D / 8)
@@ -1092,7 +1127,7 @@ paged_attn_kernel(const __grid_constant__ CUtensorMap tmap, const __grid_constan
             }
             fence_proxy_async_smem();
             __syncwarp();
-            if (more && lane == 0) issue_half<D>(&tmap, a, T, rows, cu0, uu + kStages, 1, smem_u32(Vs), bv, policy);
+            if (more && lane == 0) issue_half<D>(&tmap, a, ur, 1, smem_u32(Vs), bv, policy);
             ++consumed;
         }
 
