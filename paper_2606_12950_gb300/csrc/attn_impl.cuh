@@ -11,42 +11,48 @@
 //   unit  = one tile of one (sequence, KV head) run: 16 tokens at d = 128,
 //           32 at d = 64 (kUnit), 8 KB of K and V either way; a run of n
 //           tokens has ceil(n/kUnit) units; units are ordered (s, g, tile).
-//   part  = one of NP = P * 8 equal contiguous unit ranges [i*W/NP,
-//           (i+1)*W/NP), one per warp of the P resident CTAs: every warp
-//           streams the same number of bytes (+-1 tile) whatever the length
-//           distribution.
-//   piece = the part of one run inside one part.  A run covered by one part
+//   part  = a contiguous unit range: the units are cut into equal ranges, one
+//           per resident CTA, and each of those into equal ranges, one per
+//           warp: every warp streams the same number of bytes (+-2 tiles)
+//           whatever the length distribution.  A part is a warp's range, or
+//           with MERGE a CTA's.
+//   piece = the units of one run in one warp's range.  A run inside one part
 //           is finished in place; a run cut by part boundaries leaves one
 //           fp32 partial (max, sum, unnormalised output) per part, which the
-//           combine kernel below merges in part order.
-// Inside a CTA each of the 8 warps is one part of that split: it streams its
-// own contiguous range of units through its own shared-memory stage, issuing
-// its own 2-D TMA loads (128-byte swizzle) of each unit's K and V tiles with
-// one mbarrier for K and one for V: the next unit's K streams in while the
-// warp does softmax and P.V on the current one, the next V while it does the
-// next q.K.  (Measured on GB300: one issuing thread per SM cannot keep HBM
-// busy with these 2 KB boxes; one per warp can.)  The pool rows of a warp's
-// units are resolved from the block table in the prologue, while the memory
-// system is idle, so no table load sits on the streaming path, and each
-// run's q rows (and, for the run's last tile, this step's new K/V rows) are
-// staged into the warp's shared buffers by cp.async one piece ahead.  A run
-// that ends inside a warp's range is written out by that warp directly; no
-// state is merged between warps of a CTA.
+//           combine kernel below merges in part order, a CTA's partials
+//           first.
+// Each warp streams its own contiguous range of units through its own
+// shared-memory stage, issuing its own 2-D TMA loads (128-byte swizzle) of
+// each unit's K and V tiles with one mbarrier for K and one for V: the next
+// unit's K streams in while the warp does softmax and P.V on the current one,
+// the next V while it does the next q.K.  (Measured on GB300: one issuing
+// thread per SM cannot keep HBM busy with these 2 KB boxes; one per warp
+// can.)  The pool rows of a warp's units are resolved from the block table in
+// the prologue, while the memory system is idle, so no table load sits on the
+// streaming path, and each run's q rows (and, for the run's last tile, this
+// step's new K/V rows) are staged into the warp's shared buffers by cp.async
+// one piece ahead.
 //
-// Small batches (MERGE, chosen by attn_run): a part is a CTA's range of units,
-// cut again into one range per warp.  What bounds them is latency: a warp
-// takes its units one after another, and each part's record is one more for
-// the combine to fetch.  So the units go to as many warps as there are (one
-// unit a warp at least, instead of 64 tokens), and the warps of a CTA that
-// share a run merge their states in shared memory: the CTA leaves the run's
-// output, or one record for the combine instead of six.  One sequence of 8193
-// tokens (32 q / 8 KV heads, 33.6 MB) has 38 records a run instead of 128;
-// a step took 18.0 us before and 14.4 now (of it, the combine's column slices
-// below: 2.3); 8 sequences of 601-3500 tokens (40 q / 8 KV heads, 67 MB) 20.9
-// and 19.9.  The line at 8 units a warp: with the merge at every size the
-// 64-sequence batch (29 units a warp) took 72.9 us against 72.2, because
-// every CTA then waits for its slowest warp; at 4 units instead of 8 the 8
-// sequences (4.5 units a warp) took 21.1 us against 20.3.
+// MERGE: the warps of a CTA that share a run merge their states in shared
+// memory at the CTA's end, so that the CTA leaves the run's output, or one
+// record instead of six.  The combine then has far fewer records to fetch, at
+// the cost of a barrier and the merge (about 1 us) at the end of every CTA.
+// - Without step overlap the combine is on the critical path, and the merge
+//   pays at every size.  Same box, merged and not: 48 sequences at 8 query
+//   heads a KV head 76.4 and 77.9 us, three co-located models 266.6 and
+//   275.6, the 64-sequence layer 69.0 and 71.2, 1024 long contexts 690.3 and
+//   695.7.
+// - Where the next step's decode kernel overlaps the combine (chain 3), only
+//   the CTAs' later end shows: 69.8 and 68.1 us for the 64-sequence layer.
+//   There each warp leaves its record.  The bits are the same: the combine
+//   merges a CTA's records in the same order and arithmetic first.
+// - Small batches always merge (kMergeUnits).  What bounds them is latency: a
+//   warp takes its units one after another, and every record is one more to
+//   fetch, so their units go to as many warps as there are.  One sequence of
+//   8193 tokens (32 q / 8 KV heads, 33.6 MB) has 38 records a run instead of
+//   128; a step took 18.0 us before and 14.4 after (of it, the combine's
+//   column slices: 2.3).  8 sequences of 601-3500 tokens (40 q / 8 KV heads,
+//   67 MB, 4.5 units a warp): 20.3 us, 21.1 with the line at 4 units.
 //
 // Grid-to-grid order: the kernel is launched as a programmatic dependent.
 // Alone it releases the next grid and waits for the one before; as part of
@@ -67,6 +73,7 @@
 //                operand layout with movmatrix.
 #pragma once
 
+#include <algorithm>
 #include <cstdint>
 
 #include <cuda.h>
@@ -102,7 +109,8 @@ constexpr int kSub = kUnit<D> / kTile;            // boxes' rows per unit
 // a part's least tokens (4 units at d = 128, 2 at d = 64): with 128 at d = 64
 // a step of four short sequences took 18.5 us instead of 15.5
 constexpr int kMinPartTokens = 64;
-// Below this many units a warp the parts are CTAs (MERGE): see the kernel.
+// Below this many units a warp (by the table's width) a warp may have a single
+// unit and the CTAs merge in every mode.
 constexpr int kMergeUnits = 8;
 constexpr uint32_t kHalfBytes = kTile * 128;      // one 64-column box: 16 rows x 128 B
 constexpr uint64_t kWaitLimitNs = 2000000000ull;  // bounded mbarrier waits: 2 s
@@ -134,7 +142,7 @@ struct AttnArgs {
     const int32_t *ctx_lens;
     int32_t *err;
     float *ws_part;
-    int2 *ws_run;            // per run: (first part, parts) if split, else (part, 0)
+    int2 *ws_run;            // per run: the parts of its records, [x, y); y = x if it has none
     int64_t rows_per_page;   // page_bytes / (d * 2)
     int64_t pool_pages;
     int32_t pages_per_block;
@@ -145,7 +153,8 @@ struct AttnArgs {
     int32_t bs_shift;        // log2(bs), or -1
     int32_t rows_cap;        // boxes whose pool rows are resolved up front
     int32_t P;               // CTAs
-    int32_t nwarps;          // warps per CTA (<= kWarps), one part each
+    int32_t nwarps;          // warps per CTA (<= kWarps)
+    int32_t min_units;       // least units of a warp (but in a CTA with fewer units than warps)
     float qk_scale;          // scale * log2(e)
     // shared-prefix (cascade) mode: tokens of each sequence's prefix handled
     // by the prefix kernel ([S], multiples of 16; null = none), its records
@@ -751,12 +760,6 @@ __device__ __forceinline__ int32_t unit_row(const AttnArgs &a, const int32_t *T,
     return (int32_t)((int64_t)phys * a.rows_per_page + (tok0 - blk * a.bs) + (int64_t)r.g * a.bs);
 }
 
-// the part (of NP) whose range contains unit u
-__device__ __forceinline__ int32_t part_of(int64_t u, int64_t W, int64_t P)
-{
-    return (int32_t)(((u + 1) * P - 1) / W);
-}
-
 // per-part partial: o[G][D], m[G], l[G], padded to a multiple of 4 floats so
 // every record starts 16-byte aligned
 template <int D, int G>
@@ -770,11 +773,12 @@ __device__ __forceinline__ void merge_record(float &M, float &L, float4 &O, floa
     if (m == -INFINITY) return;
     const float Mn = fmaxf(M, m);
     const float sa = fast_exp2(M - Mn), sb = fast_exp2(m - Mn);
-    L = L * sa + l * sb;
-    O.x = O.x * sa + o.x * sb;
-    O.y = O.y * sa + o.y * sb;
-    O.z = O.z * sa + o.z * sb;
-    O.w = O.w * sa + o.w * sb;
+    // spelled out, so that every kernel that merges rounds alike
+    L = __fmaf_rn(L, sa, __fmul_rn(l, sb));
+    O.x = __fmaf_rn(O.x, sa, __fmul_rn(o.x, sb));
+    O.y = __fmaf_rn(O.y, sa, __fmul_rn(o.y, sb));
+    O.z = __fmaf_rn(O.z, sa, __fmul_rn(o.z, sb));
+    O.w = __fmaf_rn(O.w, sa, __fmul_rn(o.w, sb));
     M = Mn;
 }
 
@@ -973,37 +977,43 @@ paged_attn_kernel(const __grid_constant__ CUtensorMap tmap, const __grid_constan
         __syncthreads();
     }
 
-    // The W units are cut into NP = min(P * NW, W) equal parts; part i is
-    // [i*W/NP, (i+1)*W/NP) and belongs to warp i % NW of CTA i / NW (with
-    // MERGE to CTA i, at least NW units each).
-    // With NP <= W every part is non-empty, so a run's contributors are
-    // exactly the parts part_of(first unit) .. part_of(last unit).  A part
-    // gets at least MIN_UNITS units when the batch is small (fewer
-    // partials to write and merge; enough warps still stream to fill HBM).
+    // The W units are cut into NC equal ranges, one per CTA, and a CTA's range
+    // into equal ranges, one per warp: a warp gets at least a.min_units units
+    // when the batch is small (fewer partials to write and merge; enough warps
+    // still stream to fill HBM).  The parts are the warps' ranges, numbered
+    // blockIdx * NW + warp, or with MERGE the CTAs' ranges.  Every part is
+    // non-empty, and a run's contributors are exactly the parts from its
+    // first unit's to its last unit's.
     const int32_t W = T[S];
-    constexpr int MIN_UNITS = kMinPartTokens / UNIT;
-    const int32_t most = MERGE ? a.P : a.P * NW;
-    const int32_t fine = MERGE ? (W + NW - 1) / NW : W / MIN_UNITS > 0 ? W / MIN_UNITS : W;
-    const int32_t NP = fine < most ? fine : most;
-    const int32_t first_part = MERGE ? (int32_t)blockIdx.x : (int32_t)blockIdx.x * NW;
-    const int32_t part = MERGE ? first_part : first_part + warp;
-    if ((MERGE ? first_part : part) >= NP) {  // no CTA-wide barrier below this point without MERGE
+    const int32_t fine = a.min_units > 1 ? W / (NW * a.min_units) : (W + NW - 1) / NW;
+    const int32_t NC = W > 0 ? min(max(fine, 1), a.P) : 0;
+    const int32_t bid = (int32_t)blockIdx.x;
+    if (bid >= NC) {
         if (chained) grid_dependency_wait();
         return;
     }
-    // first unit of part p: p * W / NP, with W = wq * NP + wr
-    const int32_t wq = (int32_t)((uint32_t)W / (uint32_t)NP), wr = W - wq * NP;
-    const float np_inv = inv_of(NP);
-    auto part_begin = [&](int32_t p) {
-        return NP < 65536 / 2 ? p * wq + div_est((uint32_t)p * (uint32_t)wr, (uint32_t)NP, np_inv)
-                              : (int32_t)((int64_t)p * W / NP);
+    // first unit of CTA i: i * W / NC, with W = wq * NC + wr
+    const int32_t wq = (int32_t)((uint32_t)W / (uint32_t)NC), wr = W - wq * NC;
+    const float nc_inv = inv_of(NC);
+    auto cta_begin = [&](int32_t i) {
+        return NC < 32768 ? i * wq + div_est((uint32_t)i * (uint32_t)wr, (uint32_t)NC, nc_inv)
+                          : (int32_t)((int64_t)i * W / NC);
     };
-    const int32_t g0 = part_begin(part), g1 = part_begin(part + 1);  // this part's units
-    const int32_t cu0 = MERGE ? g0 : part_begin(first_part);         // this CTA's first
-    const int32_t nu = g1 - g0;
-    // this warp's units: the part's without MERGE
-    const int32_t u0 = MERGE ? g0 + warp * nu / NW : g0;
-    const int32_t u1 = MERGE ? g0 + (warp + 1) * nu / NW : g1;
+    const int32_t cu0 = cta_begin(bid), cu1 = cta_begin(bid + 1), nu = cu1 - cu0;  // this CTA's units
+    const int32_t nw = min(NW, nu);  // warps with units (all but where W < NW)
+    if (!MERGE && warp >= nw) {  // no CTA-wide barrier below this point without MERGE
+        if (chained) grid_dependency_wait();
+        return;
+    }
+    // this warp's units
+    const int32_t nq = (int32_t)((uint32_t)nu / (uint32_t)nw), nr = nu - nq * nw;
+    const float nw_inv = inv_of(nw);
+    auto warp_begin = [&](int w) {  // w * nu / nw
+        return w < nw ? cu0 + w * nq + div_est((uint32_t)(w * nr), (uint32_t)nw, nw_inv) : cu1;
+    };
+    const int32_t u0 = warp_begin(warp), u1 = warp_begin(warp + 1);
+    const int32_t part = MERGE ? bid : bid * NW + warp;
+    const int32_t g0 = MERGE ? cu0 : u0, g1 = MERGE ? cu1 : u1;  // this part's units
 
     // ---- prologue 2: resolve the block table for this warp's units while the
     // memory system is idle (later lookups would queue behind the TMA stream)
@@ -1013,11 +1023,7 @@ paged_attn_kernel(const __grid_constant__ CUtensorMap tmap, const __grid_constan
         __syncwarp();
     }
     float *mbuf = reinterpret_cast<float *>(mbufs) + (size_t)warp * MF;
-    if (MERGE && lane == 0) {
-        chains[warp].x = -1;
-        if (u0 == u1)  // no units: nothing to merge from this warp
-            for (int h = 0; h < G; ++h) mbuf[G * D + h] = -INFINITY;
-    }
+    if (MERGE && lane == 0) chains[warp].x = -1;
 
     const uint64_t policy = l2_policy_evict_first();
     // stage st of this warp: its K and V tiles and their barriers
@@ -1135,8 +1141,10 @@ paged_attn_kernel(const __grid_constant__ CUtensorMap tmap, const __grid_constan
         const int32_t r = run.s * Hkv + run.g;
         // a run whose prefix lives in prefix records always leaves a partial
         const bool split = run.begin < g0 || run_end > g1 || skip > 0;
-        // parts of the run that starts in this one (told to the combine)
-        auto parts = [&]() { return !split ? 0 : run_end > g1 ? part_of(run_end - 1, W, NP) - part + 1 : 1; };
+        // the run's first part and its last one tell the combine where its
+        // records begin and end
+        const bool first = run.begin >= g0, last = run_end <= g1;
+        const int end = split ? part + 1 : part;
         uint16_t *orow = a.out + ((int64_t)run.s * Hq + (int64_t)run.g * G) * D;
         float *slot = a.ws_part + ((int64_t)r + part) * MF;
         // (MERGE) the part's share of the run; it may go on over several warps
@@ -1144,15 +1152,18 @@ paged_attn_kernel(const __grid_constant__ CUtensorMap tmap, const __grid_constan
         if (!MERGE || (u == lo && pe == hi)) {
             make_ready();
             comp.store(orow, slot, split, lane);
-            if (run.begin >= g0 && lane == 0)  // each run has one first part: it tells the combine
-                a.ws_run[r] = make_int2(part, parts());
+            if (lane == 0) {
+                if (first) a.ws_run[r].x = part;
+                if (last) a.ws_run[r].y = end;
+            }
         } else if (u != lo) {  // goes on from an earlier warp, whose chain merges it
             comp.store(nullptr, mbuf, true, lane);
         } else {  // goes on in the next warp: the last piece here, so the stage is free
             comp.store(nullptr, reinterpret_cast<float *>(wstage), true, lane);
+            int e = warp;
+            while (warp_begin(e + 1) < hi) ++e;
             if (lane == 0)
-                chains[warp] = make_int4(r, ((hi - g0) * NW - 1) / nu - warp, run.begin >= g0 ? 1 : 0,
-                                         run.begin >= g0 || !split ? parts() : 1);
+                chains[warp] = make_int4(r, e - warp, (first ? 1 : 0) | (last ? 2 : 0), split ? 1 : 0);
         }
         u = pe;
         run = next;
@@ -1186,7 +1197,8 @@ paged_attn_kernel(const __grid_constant__ CUtensorMap tmap, const __grid_constan
                     slot[G * D + G + h] = L;
                 }
             }
-            if (c == 0 && ch.z) a.ws_run[ch.x] = make_int2(part, ch.w);
+            if (c == 0 && (ch.z & 1)) a.ws_run[ch.x].x = part;
+            if (c == 0 && (ch.z & 2)) a.ws_run[ch.x].y = part + ch.w;
         }
     }
     if (chained) grid_dependency_wait();
@@ -1205,7 +1217,7 @@ paged_attn_kernel(const __grid_constant__ CUtensorMap tmap, const __grid_constan
 // the attention kernel return at once.
 struct CombineArgs {
     uint16_t *out;
-    const int2 *ws_run;    // per run: (first part, parts), parts = 0 when not split
+    const int2 *ws_run;    // per run: the parts of its records, [x, y); y = x when not split
     const float *ws_part;
     int32_t S;
     int32_t Hkv;
@@ -1215,12 +1227,12 @@ struct CombineArgs {
 };
 
 constexpr int kCombineMaxThreads = 1024;
-constexpr int kCombineBatch = 8;  // records each thread loads per round trip
+constexpr int kCombineBatch = 8;  // records each thread loads per round trip, with few runs
 
 // CTAs per run (CS) and thread groups per combine CTA.
 //
-// Where each run has a CTA (CS = 1; kCombineBatch loads in flight per
-// thread): enough groups for about 8 records per thread, up to 1024 threads,
+// Where each run has a CTA (CS = 1; six loads in flight per thread, which 64
+// registers hold): enough groups for about 8 records per thread, up to 1024 threads,
 // and at least 128 threads (one group when a run's output has 128 float4
 // columns or more).  Small CTAs leave room on the SMs for the next step's
 // decode CTAs, which start as the combine's CTAs finish: on the
@@ -1243,7 +1255,7 @@ inline int combine_groups(double records_per_run)
     constexpr int NC = G * D / 4 / CS;
     constexpr int floor_threads = CS == 1 ? 128 : 64;
     const int base = NC >= floor_threads ? 1 : floor_threads / NC;
-    const int most = CS == 1 ? kCombineMaxThreads / NC : (16 > base ? 16 : base);
+    const int most = CS == 1 ? kCombineMaxThreads / NC : std::max(base, std::min(16, kCombineMaxThreads / 2 / NC));
     int want = (int)(records_per_run / 8.0 + 0.999);
     return want < base ? base : (want > most ? most : want);
 }
@@ -1259,9 +1271,9 @@ template <int D, int G, int CPT, int CS = 1>
 struct CombineShape {
     static constexpr int NC = G * D / 4 / CS;  // float4 columns of a CTA: a CS-th of a run's output
     static constexpr int NCT = NC / CPT;   // threads of a group
-    static constexpr int MAX_THREADS = CPT == 1 ? kCombineMaxThreads : NCT;
+    static constexpr int MAX_THREADS = CPT > 1 ? NCT : CS == 1 ? kCombineMaxThreads : kCombineMaxThreads / 2;
     static constexpr int MIN_CTAS = CPT == 1 ? 1 : 28 / ((NCT + 31) / 32);  // 28 warps an SM: 72 registers
-    static constexpr int BATCH = CPT == 1 ? kCombineBatch : 4;
+    static constexpr int BATCH = CPT > 1 ? 4 : CS == 1 ? 6 : kCombineBatch;
 };
 
 // shared memory of a CTA of `threads` threads: the groups' states for the
@@ -1272,7 +1284,7 @@ inline size_t combine_smem_bytes(int threads)
     return threads > CombineShape<D, G, CPT, CS>::NCT ? (size_t)threads * CPT * (2 * sizeof(float) + sizeof(float4)) : 0;
 }
 
-template <int D, int G, int CPT, int CS>
+template <int D, int G, int CPT, int CS, bool WARPS>
 __global__ void __launch_bounds__(CombineShape<D, G, CPT, CS>::MAX_THREADS, CombineShape<D, G, CPT, CS>::MIN_CTAS)
 combine_kernel(const __grid_constant__ CombineArgs c)
 {
@@ -1293,7 +1305,7 @@ combine_kernel(const __grid_constant__ CombineArgs c)
     const int2 info = c.ws_run[r];
     const int s = r / c.Hkv, g = r % c.Hkv;
     const int npre = (c.skip != nullptr && c.skip[s] > 0) ? c.KS : 0;
-    const int cnt = info.y + npre;
+    const int cnt = info.y - info.x + npre;
     if (cnt == 0) return;  // finished inside the attention kernel (or empty)
     const float *base = c.ws_part + ((int64_t)r + info.x) * MF;
     uint16_t *orow = c.out + ((int64_t)s * c.Hkv * G + (int64_t)g * G) * D;
@@ -1315,30 +1327,60 @@ combine_kernel(const __grid_constant__ CombineArgs c)
         L[j] = 0.f;
         O[j] = make_float4(0.f, 0.f, 0.f, 0.f);
     }
-    for (int k0 = grp; k0 < cnt; k0 += NG * B) {
-        float mv[B][CPT], lv[B][CPT];
-        float4 ov[B][CPT];
+    // record k: prefix record k, or, past those, the suffix's (r = s * Hkv + g)
+    auto record = [&](int k) {
+        return k < npre ? c.ws_pre + ((int64_t)k * (int)gridDim.x + r) * MF : base + (int64_t)(k - npre) * MF;
+    };
+    if constexpr (!WARPS) {
+        for (int k0 = grp; k0 < cnt; k0 += NG * B) {
+            float mv[B][CPT], lv[B][CPT];
+            float4 ov[B][CPT];
 #pragma unroll
-        for (int b = 0; b < B; ++b) {
-            const int k = k0 + b * NG;
+            for (int b = 0; b < B; ++b) {
+                const int k = k0 + b * NG;
 #pragma unroll
-            for (int j = 0; j < CPT; ++j) mv[b][j] = -INFINITY;
-            if (k < cnt) {
-                const float *sl = k < npre ? c.ws_pre + (((int64_t)k * c.S + s) * c.Hkv + g) * MF
-                                           : base + (int64_t)(k - npre) * MF;
+                for (int j = 0; j < CPT; ++j) mv[b][j] = -INFINITY;
+                if (k < cnt) {
+                    const float *sl = record(k);
 #pragma unroll
-                for (int j = 0; j < CPT; ++j) {
-                    mv[b][j] = sl[G * D + h[j]];
-                    lv[b][j] = sl[G * D + G + h[j]];
-                    ov[b][j] = *reinterpret_cast<const float4 *>(sl + col[j] * 4);
+                    for (int j = 0; j < CPT; ++j) {
+                        mv[b][j] = sl[G * D + h[j]];
+                        lv[b][j] = sl[G * D + G + h[j]];
+                        ov[b][j] = *reinterpret_cast<const float4 *>(sl + col[j] * 4);
+                    }
                 }
             }
+#pragma unroll
+            for (int b = 0; b < B; ++b)
+#pragma unroll
+                for (int j = 0; j < CPT; ++j) merge_record(M[j], L[j], O[j], mv[b][j], lv[b][j], ov[b][j]);
         }
+    } else {
+        // a record per warp: those of a CTA are merged first, as the CTA itself
+        // does when it merges them (MERGE), so that both ways give the same bits
+        static_assert(CPT == 1, "no shared prefix: its decode CTAs have kWarps warps");
+        constexpr int CW = kPlainWarps;
+        const int first = info.x;
+        for (int b0 = (first / CW + grp) * CW; b0 < info.y; b0 += NG * CW) {
+            float mv[CW], lv[CW];
+            float4 ov[CW];
 #pragma unroll
-        for (int b = 0; b < B; ++b)
+            for (int b = 0; b < CW; ++b) {
+                const int p = b0 + b;
+                mv[b] = -INFINITY;
+                if (p >= first && p < info.y) {
+                    const float *sl = base + (int64_t)(p - first) * MF;
+                    mv[b] = sl[G * D + h[0]];
+                    lv[b] = sl[G * D + G + h[0]];
+                    ov[b] = *reinterpret_cast<const float4 *>(sl + col[0] * 4);
+                }
+            }
+            float Mc = -INFINITY, Lc = 0.f;
+            float4 Oc = make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
-            for (int j = 0; j < CPT; ++j)
-                merge_record(M[j], L[j], O[j], mv[b][j], lv[b][j], ov[b][j]);
+            for (int b = 0; b < CW; ++b) merge_record(Mc, Lc, Oc, mv[b], lv[b], ov[b]);
+            merge_record(M[0], L[0], O[0], Mc, Lc, Oc);
+        }
     }
     if (NG > 1) {
         const int nt = (int)blockDim.x;

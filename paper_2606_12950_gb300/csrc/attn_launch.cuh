@@ -47,16 +47,28 @@ int cached_occupancy(Fn fn, int threads, size_t smem, int *occ, OccCache &c)
 }
 
 // The combine over c's runs: `groups` thread groups a CTA, CS CTAs a run.
-template <int D, int G, int CPT, int CS>
+template <int D, int G, int CPT, int CS, bool WARPS>
 int combine_launch(const CombineArgs &c, int groups, cudaLaunchConfig_t cfg)
 {
     const int threads = groups * CombineShape<D, G, CPT, CS>::NCT;
     cfg.gridDim = dim3((unsigned)(c.S * c.Hkv), (unsigned)CS);
     cfg.blockDim = dim3((unsigned)threads);
     cfg.dynamicSmemBytes = combine_smem_bytes<D, G, CPT, CS>(threads);
-    if (cudaLaunchKernelEx(&cfg, combine_kernel<D, G, CPT, CS>, c) != cudaSuccess) return KV_ERR_CUDA;
+    if (cudaLaunchKernelEx(&cfg, combine_kernel<D, G, CPT, CS, WARPS>, c) != cudaSuccess) return KV_ERR_CUDA;
     kvp_note_stream(cfg.stream, true);
     return KV_OK;
+}
+
+// Few runs: each run's columns spread over CS CTAs (kSlicedCtas).
+template <int D, int G, bool WARPS>
+int combine_run(const CombineArgs &c, double per_run, int sm_count, const cudaLaunchConfig_t &cfg)
+{
+    const int runs = c.S * c.Hkv;
+    if (8 * runs <= kSlicedCtas * sm_count)
+        return combine_launch<D, G, 1, 8, WARPS>(c, combine_groups<D, G, 8>(per_run), cfg);
+    if (4 * runs <= kSlicedCtas * sm_count)
+        return combine_launch<D, G, 1, 4, WARPS>(c, combine_groups<D, G, 4>(per_run), cfg);
+    return combine_launch<D, G, 1, 1, WARPS>(c, combine_groups<D, G, 1>(per_run), cfg);
 }
 
 // what: kLaunchQuery (only *P_out), kLaunchBoth (attention, then combine),
@@ -90,25 +102,32 @@ int attn_run(const CUtensorMap *tmap, AttnArgs a, int P_req, int sm_count, cudaS
     for (int k = 4; k < 31; ++k)
         if (a.bs == 1 << k) a.bs_shift = k;
     a.P = P;
-    // A batch whose table has room for fewer than kMergeUnits units a warp
-    // runs with its CTAs as the parts (MERGE), if the merge's buffers cost no
-    // CTA per SM.  The rule sees the table's width, not the lengths, so that
-    // a call gives the same bits whether the lengths come with it or not.
-    int parts_per_cta = a.nwarps;
+    // Where the table has room for fewer than kMergeUnits units a warp, warps
+    // may have a single unit and the CTAs merge their warps' records (MERGE).
+    // This rule sees the table's width, not the lengths, so that a call gives
+    // the same bits whether the lengths come with it or not.  Larger batches
+    // merge too, unless the next step's decode kernel overlaps the combine
+    // (chain 3): then only the CTAs' later end shows.  The bits are the same
+    // either way (CombineArgs::per_cta).  Beside a shared prefix only the
+    // first rule holds.  In no case if the buffers cost a CTA per SM.
     const int64_t most_units =
         (int64_t)a.S * a.Hkv * (((int64_t)a.max_blocks * a.bs + kUnit<D> - 1) / kUnit<D>);
-    if (most_units < (int64_t)kMergeUnits * P * a.nwarps) {
+    const bool small = most_units < (int64_t)kMergeUnits * P * a.nwarps;
+    bool merge = false;
+    a.min_units = kMinPartTokens / kUnit<D>;
+    if (small || (a.chain != 3 && a.skip == nullptr)) {
         const size_t smem_merge = attn_smem_bytes<D, G>(a.S, kRowsCap, a.nwarps, true);
         int occ_merge = 0;
         static OccCache merge_cache;
         if (smem_merge <= kSmemMax) {
             if (cached_occupancy(fn_merge, a.nwarps * 32, smem_merge, &occ_merge, merge_cache) != KV_OK)
                 return KV_ERR_CUDA;
-            if (occ_merge >= occ) {
-                fn = fn_merge;
-                smem = smem_merge;
-                parts_per_cta = 1;
-            }
+            merge = occ_merge >= occ;
+        }
+        if (merge) {
+            fn = fn_merge;
+            smem = smem_merge;
+            if (small) a.min_units = 1;
         }
     }
     // both kernels are programmatic dependents of what precedes them in the
@@ -131,19 +150,19 @@ int attn_run(const CUtensorMap *tmap, AttnArgs a, int P_req, int sm_count, cudaS
     if (what == kLaunchAttention) return KV_OK;
     CombineArgs c{a.out, a.ws_run, a.ws_part, a.S, a.Hkv, a.skip, a.ws_pre, a.KS};
     cudaLaunchConfig_t ccfg = cfg;
-    // records per run: at most one per part, spread over the runs, plus the
-    // prefix records in shared-prefix mode
+    // records per run (of warps; a CTA's if warps may have a single unit):
+    // at most one per part, spread over the runs, plus the prefix records in
+    // shared-prefix mode
     const int runs = a.S * a.Hkv;
-    const double per_run = (double)P * parts_per_cta / std::max(1, runs) + 1.0 + (a.skip ? a.KS : 0);
+    const double per_run = (double)P * (a.min_units == 1 ? 1 : a.nwarps) / std::max(1, runs) + 1.0 + (a.skip ? a.KS : 0);
     if constexpr (G * D / 4 >= 128) {
         // one group in shared-prefix mode: two columns a thread, so that
         // every member run fits in one wave
-        if (a.skip != nullptr && combine_groups<D, G, 1>(per_run) == 1) return combine_launch<D, G, 2, 1>(c, 1, ccfg);
+        if (a.skip != nullptr && combine_groups<D, G, 1>(per_run) == 1)
+            return combine_launch<D, G, 2, 1, false>(c, 1, ccfg);
     }
-    // few runs: each run's columns spread over CS CTAs (kSlicedCtas)
-    if (8 * runs <= kSlicedCtas * sm_count) return combine_launch<D, G, 1, 8>(c, combine_groups<D, G, 8>(per_run), ccfg);
-    if (4 * runs <= kSlicedCtas * sm_count) return combine_launch<D, G, 1, 4>(c, combine_groups<D, G, 4>(per_run), ccfg);
-    return combine_launch<D, G, 1, 1>(c, combine_groups<D, G, 1>(per_run), ccfg);
+    return merge || a.skip != nullptr ? combine_run<D, G, false>(c, per_run, sm_count, ccfg)
+                                      : combine_run<D, G, true>(c, per_run, sm_count, ccfg);
 }
 
 // Shared-prefix kernel: with launch = false only reports the CTAs that fit

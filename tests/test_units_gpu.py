@@ -177,3 +177,34 @@ def test_key_splits_of_a_shared_prefix(tokens, G, Hkv, d):
     assert np.array_equal(pool.download(), ref_pool)
     _check(db.out_f64(), oracle.batch_attention(b, pool=ref_pool), (tokens, G))
     assert pool.error() == 0
+
+
+@pytest.mark.parametrize("lens", MERGE_LENS.values(), ids=MERGE_LENS.keys())
+@pytest.mark.parametrize("G,Hkv,d,variant", [(1, 4, 128, 2), (4, 8, 128, 2), (8, 1, 128, 2), (4, 2, 64, 2), (4, 2, 64, 1)])
+def test_records_per_warp_and_per_cta_give_the_same_bits(G, Hkv, d, variant, lens):
+    """A table too wide for the small-batch rule: alone a call merges its warps'
+    records in the CTAs, after another call's combine (step overlap) it leaves
+    them to the combine.  The same bits, also with fewer units than warps, with
+    one CTA and with several."""
+    from paper_2606_12950_gb300.runner import DeviceBatch, DevicePool
+
+    b = W.make_batch(7500 + G + d, lens, Hq=G * Hkv, Hkv=Hkv, d=d, bs=16, extra_blocks=3)
+    wide = np.full((b.S, 16384), -1, np.int32)
+    wide[:, : b.max_blocks] = b.table
+    b.table, b.max_blocks = wide, 16384
+    pool = DevicePool(b.n_pages, b.page_elems * 2, b.bs, [(b.Hkv, b.d)])
+    pool.upload(b.pool)
+    pool.set_variant(variant)
+    for splits in (0, 1, 3):
+        db = DeviceBatch(pool, 0, b, splits)
+        db.append_attend()
+        torch.cuda.synchronize()
+        alone = db.out_bits()
+        pool.set_step_overlap(True)
+        for _ in range(3):
+            db.append_attend()
+        torch.cuda.synchronize()
+        pool.set_step_overlap(False)
+        assert np.array_equal(alone, db.out_bits()), splits
+    _check(db.out_f64(), oracle.batch_attention(b, pool=oracle.batch_append(b)), (G, Hkv, d))
+    assert pool.error() == 0
