@@ -782,6 +782,32 @@ __device__ __forceinline__ void merge_record(float &M, float &L, float4 &O, floa
     M = Mn;
 }
 
+// The records of one CTA's warps (m = -inf: none) as one state, for one float4
+// column: the maximum first, so that the sums wait on no chain of rescales
+// (one long sequence 14.2 -> 13.9 us a step, 8 sequences 19.3 -> 19.1, 48
+// with 8 query heads a KV head 77.3 -> 76.8, against one record at a time).
+// The CTAs (MERGE) and the combine both use it: the same bits.
+template <int N>
+__device__ __forceinline__ void merge_group(float &M, float &L, float4 &O, const float (&m)[N], const float (&l)[N],
+                                            const float4 (&o)[N])
+{
+    M = m[0];
+#pragma unroll
+    for (int k = 1; k < N; ++k) M = fmaxf(M, m[k]);
+    L = 0.f;
+    O = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+    for (int k = 0; k < N; ++k) {
+        if (m[k] == -INFINITY) continue;
+        const float e = fast_exp2(m[k] - M);
+        L = __fmaf_rn(l[k], e, L);
+        O.x = __fmaf_rn(o[k].x, e, O.x);
+        O.y = __fmaf_rn(o[k].y, e, O.y);
+        O.z = __fmaf_rn(o[k].z, e, O.z);
+        O.w = __fmaf_rn(o[k].w, e, O.w);
+    }
+}
+
 // a merged column's four outputs, bf16(O / L)
 __device__ __forceinline__ void store_column(uint16_t *dst, const float4 &O, float L)
 {
@@ -1179,13 +1205,23 @@ paged_attn_kernel(const __grid_constant__ CUtensorMap tmap, const __grid_constan
             const int w = i / NC, c = i % NC, h = c * 4 / D;
             const int4 ch = chains[w];
             if (ch.x < 0) continue;
-            float M = -INFINITY, L = 0.f;
-            float4 O = make_float4(0.f, 0.f, 0.f, 0.f);
-            for (int k = 0; k <= ch.y; ++k) {
-                const float *rec = k == 0 ? reinterpret_cast<const float *>(stages + (size_t)w * kStages * STAGE_BYTES)
-                                          : reinterpret_cast<const float *>(mbufs) + (size_t)(w + k) * MF;
-                merge_record(M, L, O, rec[G * D + h], rec[G * D + G + h], *reinterpret_cast<const float4 *>(rec + c * 4));
+            float mv[kWarps], lv[kWarps];
+            float4 ov[kWarps];
+#pragma unroll
+            for (int k = 0; k < kWarps; ++k) {
+                mv[k] = -INFINITY;
+                if (k <= ch.y) {
+                    const float *rec = k == 0
+                                           ? reinterpret_cast<const float *>(stages + (size_t)w * kStages * STAGE_BYTES)
+                                           : reinterpret_cast<const float *>(mbufs) + (size_t)(w + k) * MF;
+                    mv[k] = rec[G * D + h];
+                    lv[k] = rec[G * D + G + h];
+                    ov[k] = *reinterpret_cast<const float4 *>(rec + c * 4);
+                }
             }
+            float M, L;
+            float4 O;
+            merge_group(M, L, O, mv, lv, ov);
             make_ready();
             if (ch.w == 0) {
                 store_column(a.out + (int64_t)ch.x * (G * D) + c * 4, O, L);
@@ -1375,10 +1411,9 @@ combine_kernel(const __grid_constant__ CombineArgs c)
                     ov[b] = *reinterpret_cast<const float4 *>(sl + col[0] * 4);
                 }
             }
-            float Mc = -INFINITY, Lc = 0.f;
-            float4 Oc = make_float4(0.f, 0.f, 0.f, 0.f);
-#pragma unroll
-            for (int b = 0; b < CW; ++b) merge_record(Mc, Lc, Oc, mv[b], lv[b], ov[b]);
+            float Mc, Lc;
+            float4 Oc;
+            merge_group(Mc, Lc, Oc, mv, lv, ov);
             merge_record(M[0], L[0], O[0], Mc, Lc, Oc);
         }
     }
