@@ -847,6 +847,15 @@ int paged_decode_attn_multi(kv_pool *p, int n, const kv_attn_batch *batches, voi
         return dispatch(it.variant, it.D, it.G, &p->tmap[it.layout], &it.a, it.P, p->sm_count, st,
                         kvp::kLaunchBoth, &P);
     }
+    // the largest first, by the room in its table: a later kernel's CTAs start as
+    // the one before frees SMs, so its CTAs' starts and ends spread as much as
+    // those of all before it; a short one last leaves that spread short work.
+    // Three co-located models (1.2, 0.3 and 0.1 GB): 273 us with the smallest
+    // first, 266 with the largest first.
+    std::stable_sort(items.begin(), items.end(), [](const MultiItem &x, const MultiItem &y) {
+        auto room = [](const MultiItem &i) { return (int64_t)i.a.S * i.a.Hkv * i.D * i.a.max_blocks; };
+        return room(x) > room(y);
+    });
     // the decode kernels as a chain (each later one starts on the SMs the one
     // before frees and waits for it at its end), then the combines
     for (size_t i = 0; i < items.size(); ++i) {
