@@ -23,8 +23,24 @@
 // softmax writes P (bf16) back over S in TMEM, and the P.V MMA reads its A
 // operand from there, so P never touches shared memory.  A CTA holds two Q
 // tiles that share every K/V tile: while one tile's four warps run the
-// softmax, the tensor core works on the other tile.  One thread issues the
-// MMAs, one warp the TMA loads, one thread owns each row.
+// softmax, the tensor core works on the other tile.  One warp issues the
+// MMAs, two the TMA loads (K's and V's), one thread owns each row.
+//
+// What paced it (SM clocks of one CTA, 128 members of two 8192-token prefixes,
+// cycles per key tile of both Q tiles, 4450 in all):
+// - the MMA issue, 70-100 cycles each from a single diverged lane: operands
+//   pass to uniform registers one by one there.  A whole warp now runs the
+//   loop and an elected lane issues: 43-56.
+// - waits of 500-1800 for the next K tile: one warp issued K's and V's boxes
+//   and 32 L2 requests a tile, one after another.  K and V now have a warp
+//   each, and ask L2 for 4 KB at a time after their loads.
+// - P is handed over in halves, so that P.V starts on the first while the
+//   second is computed.
+// Now 3390 (2048 at the tensor core's rate).  200 suffixes of about 500 tokens
+// with one 8192-token prefix 96.5 -> 82.3 us a step, 128 of about 100 with two
+// of 4096 tokens 47.0 -> 40.5, 12 of about 500 with 4096 tokens 20.2 -> 19.1.
+// Looking at four barriers at once instead of in turn gave nothing more.
+//
 // Each CTA leaves, per (sharer, KV head), one fp32 record (unnormalised o,
 // running max m, sum l) in the same format as the decode kernel's split
 // partials; the combine kernel merges prefix and suffix records, which is
@@ -42,7 +58,7 @@ constexpr int kPreKeys = 128;             // prefix tokens per pipeline tile: S'
 constexpr int kPreChunk = 64;             // granularity of prefix lengths and key splits
 constexpr int kPreStages = 2;
 constexpr int kPreSoftWarps = 4;          // per Q tile: one thread per query row
-constexpr int kPreThreads = (kPreQTiles * kPreSoftWarps + 2) * 32;  // + TMA warp + MMA warp
+constexpr int kPreThreads = (kPreQTiles * kPreSoftWarps + 3) * 32;  // + K and V load warps + MMA warp
 constexpr int kPreAhead = 4;              // key tiles asked of L2 ahead of their loads
 constexpr int kPreRowsCap = 256;          // 16-token sub-tiles resolved up front
 constexpr int kMaxKeySplits = 8;
@@ -52,6 +68,7 @@ constexpr uint32_t kPreTmemCols = 256;
 
 struct CascadeArgs {
     const uint16_t *q;
+    const uint16_t *pool;  // pool base (rows of d bf16)
     const int32_t *table;
     int32_t *err;
     float *ws_pre;        // [kMaxKeySplits][S][Hkv] records of merge_floats<D, G>() floats
@@ -110,9 +127,9 @@ struct PreSmem {
     static constexpr uint32_t Q_OFF = 0;
     static constexpr uint32_t ST_OFF = kPreQTiles * Q_TILE;
     static constexpr uint32_t BAR_OFF = ST_OFF + kPreStages * STAGE;
-    // full and empty per stage, of K and of V; per Q tile: s_full, p_full,
-    // o_done; fin; q_ready
-    static constexpr int NBARS = 4 * kPreStages + 3 * kPreQTiles + 2;
+    // full and empty per stage, of K and of V; per Q tile: s_full, p_full of
+    // each half, o_done; fin; q_ready
+    static constexpr int NBARS = 4 * kPreStages + 4 * kPreQTiles + 2;
     static constexpr uint32_t SLOT_OFF = BAR_OFF + NBARS * 8;
     static constexpr uint32_t ROWS_OFF = SLOT_OFF + 16;
     static constexpr uint32_t BYTES = ROWS_OFF + kPreRowsCap * 4;
@@ -140,10 +157,10 @@ cascade_prefix_kernel(const __grid_constant__ CUtensorMap tmap, const __grid_con
     int32_t *rows = reinterpret_cast<int32_t *>(smem + L::ROWS_OFF);
     auto bar = [&](int i) { return smem_u32(&bars[i]); };
     constexpr int FULL_K = 0, EMPTY_K = kPreStages, FULL_V = 2 * kPreStages, EMPTY_V = 3 * kPreStages;
-    constexpr int QB = 4 * kPreStages, FIN = QB + 3 * kPreQTiles, Q_READY = FIN + 1;
-    auto s_full = [&](int a) { return bar(QB + 3 * a); };
-    auto p_full = [&](int a) { return bar(QB + 3 * a + 1); };
-    auto o_done = [&](int a) { return bar(QB + 3 * a + 2); };
+    constexpr int QB = 4 * kPreStages, FIN = QB + 4 * kPreQTiles, Q_READY = FIN + 1;
+    auto s_full = [&](int a) { return bar(QB + 4 * a); };
+    auto p_full = [&](int a, int half) { return bar(QB + 4 * a + 1 + half); };  // P of keys 64 half .. 64 half + 63
+    auto o_done = [&](int a) { return bar(QB + 4 * a + 3); };
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     int bid = blockIdx.x;
@@ -156,7 +173,8 @@ cascade_prefix_kernel(const __grid_constant__ CUtensorMap tmap, const __grid_con
         for (int i = 0; i < 4 * kPreStages; ++i) mbar_init(bar(i), 1);
         for (int a = 0; a < kPreQTiles; ++a) {
             mbar_init(s_full(a), 1);
-            mbar_init(p_full(a), kPreSoftWarps * 32);
+            mbar_init(p_full(a, 0), kPreSoftWarps * 32);
+            mbar_init(p_full(a, 1), kPreSoftWarps * 32);
             mbar_init(o_done(a), 1);
         }
         mbar_init(bar(FIN), 1);
@@ -174,7 +192,7 @@ cascade_prefix_kernel(const __grid_constant__ CUtensorMap tmap, const __grid_con
     tc_fence_after();
     const uint32_t tbase = *tslot;
     bool dead = false;
-    constexpr int TMA_WARP = kPreQTiles * kPreSoftWarps, MMA_WARP = TMA_WARP + 1;
+    constexpr int LOAD_WARP = kPreQTiles * kPreSoftWarps, MMA_WARP = LOAD_WARP + 2;  // K's, V's; MMA
     // Wait for the grid before (the plan kernel; through it the table sync
     // and the previous step's combine), then release the decode kernel that
     // follows: it runs beside this grid on the SMs this grid leaves free and
@@ -243,70 +261,69 @@ cascade_prefix_kernel(const __grid_constant__ CUtensorMap tmap, const __grid_con
         mbar_arrive(bar(Q_READY));
     }
 
-    if (warp == TMA_WARP) {
-        // ---- TMA producer warp: resolves the pool rows of the CTA's key range
-        // from the block table, then streams K and V of key tile t into stage
-        // t % stages, one box per lane (one issuing thread per SM cannot keep
-        // the loads flowing) ----
+    if (warp == LOAD_WARP || warp == LOAD_WARP + 1) {
+        // ---- TMA producer warps, one of K and one of V: each resolves the pool
+        // rows of the CTA's key range from the block table (both write the same
+        // rows), then streams its half of key tile t into stage t % stages,
+        // one box per lane (one issuing thread per SM cannot keep the loads
+        // flowing; a warp's boxes are issued one after another, so that one
+        // warp for both held the next K back) ----
+        const bool is_v = warp != LOAD_WARP;
         for (int i = lane; i < min(nsub, kPreRowsCap); i += 32) rows[i] = pre_sub_row(c, lead, g, ch0 * CSUB + i);
         __syncwarp();
         const uint64_t pol = l2_policy_evict_normal();  // the prefix is re-read by every row tile
-        constexpr int NBOX = NSUB * HALVES;               // boxes of K (and of V) per full key tile
-        static_assert(2 * NBOX <= 32, "one box per lane");
-        // box (j, h): rows 16j .. 16j + 15, columns 64h .. 64h + 63 of K
-        // (lanes below NBOX) or V (from NBOX on) of a key tile
-        const bool is_v = lane >= NBOX;
-        const int j = (lane % NBOX) / HALVES, h = (lane % NBOX) % HALVES;
-        auto row_of = [&](int t) {  // of this lane's box in key tile t: -1 outside the pool
-            const int32_t q = t * NSUB + j;
+        constexpr int NBOX = NSUB * HALVES;               // boxes per full key tile
+        static_assert(NBOX <= 32, "one box per lane");
+        const int full0 = is_v ? FULL_V : FULL_K, empty0 = is_v ? EMPTY_V : EMPTY_K;
+        // box (j, h): rows 16j .. 16j + 15, columns 64h .. 64h + 63 of a key tile
+        const int j = lane / HALVES, h = lane % HALVES;
+        auto row_of = [&](int q) {  // of sub-tile q: -1 outside the pool
             const int32_t y = q < kPreRowsCap ? rows[q] : pre_sub_row(c, lead, g, ch0 * CSUB + q);
             return y < 0 ? y : y + (is_v ? c.Hkv * c.bs : 0);
         };
-        auto mine_of = [&](int t) { return lane < 2 * NBOX && t < nt && j < tile_keys(t) / kTile; };
         for (int t = 0; t < nt; ++t) {
             const int st = t % kPreStages;
-            const uint32_t par = (uint32_t)(t / kPreStages - 1) & 1u;
             const int vsub = tile_keys(t) / kTile;        // sub-tiles loaded this tile
-            const bool mine = mine_of(t);
-            const int32_t y = mine ? row_of(t) : 0;
+            const bool mine = lane < NBOX && j < vsub;
+            const int32_t y = mine ? row_of(t * NSUB + j) : 0;
             const bool ok = __all_sync(0xffffffffu, y >= 0);
-            if (!ok && lane == 0) report(c.err, KV_ERR_DEVICE_BOUNDS);
-            // the tile kPreAhead further on, into L2
-            if (mine_of(t + kPreAhead)) {
-                const int32_t ya = row_of(t + kPreAhead);
-                if (ya >= 0) tma_prefetch_2d(&tmap, h * 64, ya);
-            }
-            const uint32_t dst = sbase + L::ST_OFF + st * L::STAGE + (is_v ? L::KV_TILE : 0) + h * L::KV_HALF +
-                                 j * (kTile * 128);
-#pragma unroll
-            for (int kv = 0; kv < 2; ++kv) {
-                const uint32_t full = bar((kv ? FULL_V : FULL_K) + st);
-                if (t >= kPreStages) wait_phase(bar((kv ? EMPTY_V : EMPTY_K) + st), par, c.err, dead);
-                if (lane == 0) {
-                    if (ok)
-                        mbar_arrive_expect_tx(full, (uint32_t)vsub * HALVES * (kTile * 128));
-                    else
-                        mbar_arrive(full);  // complete the phase without data
+            const uint32_t full = bar(full0 + st);
+            if (t >= kPreStages) wait_phase(bar(empty0 + st), (uint32_t)(t / kPreStages - 1) & 1u, c.err, dead);
+            if (lane == 0) {
+                if (ok) {
+                    mbar_arrive_expect_tx(full, (uint32_t)vsub * HALVES * (kTile * 128));
+                } else {
+                    report(c.err, KV_ERR_DEVICE_BOUNDS);
+                    mbar_arrive(full);  // complete the phase without data
                 }
-                __syncwarp();
-                if (ok && mine && is_v == (kv == 1)) tma_load_2d(dst, &tmap, h * 64, y, full, pol);
+            }
+            __syncwarp();
+            if (ok && mine)
+                tma_load_2d(sbase + L::ST_OFF + st * L::STAGE + (is_v ? L::KV_TILE : 0) + h * L::KV_HALF +
+                                j * (kTile * 128),
+                            &tmap, h * 64, y, full, pol);
+            // the tile kPreAhead further on, into L2: a sub-tile's rows are
+            // consecutive in the pool
+            const int qa = (t + kPreAhead) * NSUB + lane;
+            if (lane < NSUB && qa < nsub) {
+                const int32_t ya = row_of(qa);
+                if (ya >= 0) bulk_prefetch_l2(c.pool + (int64_t)ya * D, kTile * D * 2);
             }
             __syncwarp();
         }
         // drain: the last stages' loads have landed (already waited on by the
-        // MMA thread unless a wait ran out)
+        // MMA warp unless a wait ran out)
         if (lane == 0)
-            for (int t = max(0, nt - kPreStages); t < nt; ++t) {
-                wait_phase(bar(FULL_K + t % kPreStages), (uint32_t)(t / kPreStages) & 1u, c.err, dead);
-                wait_phase(bar(FULL_V + t % kPreStages), (uint32_t)(t / kPreStages) & 1u, c.err, dead);
-            }
-    } else if (warp == MMA_WARP && lane == 0) {
+            for (int t = max(0, nt - kPreStages); t < nt; ++t)
+                wait_phase(bar(full0 + t % kPreStages), (uint32_t)(t / kPreStages) & 1u, c.err, dead);
+    } else if (warp == MMA_WARP) {
         // ---- MMA issuer.  Per Q tile a and key tile t: S_a = Q_a K_t^T into
         // TMEM, then, once the tile's warps have written P (bf16) over S,
         // O_a += P V_t with P read from TMEM.  The tensor pipe runs one
         // thread's MMAs in issue order, so S_a(t+1), issued after
         // P.V_a(t), overwrites P only after that MMA has read it.  Order:
         // S_0(0) S_1(0) | PV_0(t) S_0(t+1) PV_1(t) S_1(t+1) | ... ----
+        const uint32_t el = elect_one();
         constexpr uint32_t ID_S = idesc_bf16_f32(kPreRows, kPreKeys, 0, 0);
         constexpr uint32_t ID_S_HALF = idesc_bf16_f32(kPreRows, kPreChunk, 0, 0);
         constexpr uint32_t ID_O = idesc_bf16_f32(kPreRows, D, 0, 1);
@@ -317,42 +334,50 @@ cascade_prefix_kernel(const __grid_constant__ CUtensorMap tmap, const __grid_con
 #pragma unroll
             for (int kk = 0; kk < D / 16; ++kk)
                 umma_bf16(tbase + a * kPreTmemCols, smem_desc_sw128(qa + (kk / 4) * L::Q_HALF + (kk % 4) * 32, 16, 1024),
-                          smem_desc_sw128(ka + (kk / 4) * L::KV_HALF + (kk % 4) * 32, 16, 1024), id, kk > 0);
-            umma_commit(s_full(a));
+                          smem_desc_sw128(ka + (kk / 4) * L::KV_HALF + (kk % 4) * 32, 16, 1024), id, kk > 0, el);
+            umma_commit(s_full(a), el);
         };
-        auto issue_pv = [&](int a, int t) {
+        auto issue_pv = [&](int a, int t, int half) {
             const uint32_t va = sbase + L::ST_OFF + (t % kPreStages) * L::STAGE + L::KV_TILE;
-            const int ksteps = tile_keys(t) / 16;
-            for (int kk = 0; kk < ksteps; ++kk)
+            constexpr int STEPS = kPreChunk / 16;
+#pragma unroll
+            for (int i = 0; i < STEPS; ++i) {
+                const int kk = half * STEPS + i;
                 umma_bf16_tmem_a(tbase + a * kPreTmemCols + O_COL, tbase + a * kPreTmemCols + kk * 8,
-                                 smem_desc_sw128(va + kk * (16 * 128), L::KV_HALF, 1024), ID_O, t > 0 || kk > 0);
-            umma_commit(o_done(a));
+                                 smem_desc_sw128(va + kk * (16 * 128), L::KV_HALF, 1024), ID_O, t > 0 || kk > 0, el);
+            }
         };
         wait_phase(bar(Q_READY), 0u, c.err, dead);
         wait_phase(bar(FULL_K + 0), 0u, c.err, dead);
         tc_fence_after();
         for (int a = 0; a < kPreQTiles; ++a) issue_s(a, 0);
-        umma_commit(bar(EMPTY_K + 0));
+        umma_commit(bar(EMPTY_K + 0), el);
         for (int t = 0; t < nt; ++t) {
             const bool next = t + 1 < nt;
             for (int a = 0; a < kPreQTiles; ++a) {
                 if (a == 0)
                     wait_phase(bar(FULL_V + t % kPreStages), (uint32_t)(t / kPreStages) & 1u, c.err, dead);
-                wait_phase(p_full(a), (uint32_t)t & 1u, c.err, dead);
+                wait_phase(p_full(a, 0), (uint32_t)t & 1u, c.err, dead);
                 tc_fence_after();
-                issue_pv(a, t);
-                if (a == kPreQTiles - 1) umma_commit(bar(EMPTY_V + t % kPreStages));
+                issue_pv(a, t, 0);
+                wait_phase(p_full(a, 1), (uint32_t)t & 1u, c.err, dead);
+                if (tile_keys(t) > kPreChunk) {
+                    tc_fence_after();
+                    issue_pv(a, t, 1);
+                }
+                umma_commit(o_done(a), el);
+                if (a == kPreQTiles - 1) umma_commit(bar(EMPTY_V + t % kPreStages), el);
                 if (next) {
                     if (a == 0) wait_phase(bar(FULL_K + (t + 1) % kPreStages), (uint32_t)((t + 1) / kPreStages) & 1u,
                                            c.err, dead);
                     tc_fence_after();
                     issue_s(a, t + 1);
-                    if (a == kPreQTiles - 1) umma_commit(bar(EMPTY_K + (t + 1) % kPreStages));
+                    if (a == kPreQTiles - 1) umma_commit(bar(EMPTY_K + (t + 1) % kPreStages), el);
                 }
             }
         }
         // every MMA of this thread has completed before TMEM is released
-        umma_commit(bar(FIN));
+        umma_commit(bar(FIN), el);
         wait_phase(bar(FIN), 0u, c.err, dead);
     } else if (tid < SOFT_THREADS) {
         // ---- softmax: thread tid owns row r of Q tile qa_tile (TMEM lane r) ----
@@ -366,69 +391,67 @@ cascade_prefix_kernel(const __grid_constant__ CUtensorMap tmap, const __grid_con
             // particular P.V_a(t-1), so O is stable and P's columns are free
             wait_phase(s_full(a), (uint32_t)t & 1u, c.err, dead);
             tc_fence_after();
-            // One pass over the tile, 64 keys (one chunk) at a time: p =
-            // 2^(s * scale - m_ref) as bf16 pairs written over the first
-            // columns of S (the A operand of P.V; chunk cp's 32 words land on
-            // columns 32cp .. 32cp + 31, which hold scores already read).
-            // m_ref is the running max, raised (lazy rescale) only when a
-            // chunk exceeds it by more than 2^8: then O, l, this tile's sum
-            // and the P words already written for it are scaled by
-            // 2^(m_old - m_new) first, so every stored p stays <= 2^8 and
-            // o, l and P share one reference max.
-            float rs = 0.f;
+            // The row's maximum (scores read twice: 128 in registers spilled,
+            // 96.7 -> 123.5 us on the step above).  m_ref, the reference of o,
+            // l and P, is raised (lazy rescale) only when the tile exceeds it
+            // by more than 2^8; then O and l are scaled by 2^(m_old - m_new)
+            // first, so every stored p stays <= 2^8.
+            float mx[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
+            uint32_t v[2][32];
 #pragma unroll
-            for (int cp = 0; cp < kPreKeys / 64; ++cp) {
-                if (cp * 64 >= nk) break;
-                uint32_t v[2][32];
-                tmem_ld32(trow + cp * 64, v[0]);
-                tmem_ld32(trow + cp * 64 + 32, v[1]);
-                tmem_wait_ld();
-                float mx[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
+            for (int cp = kPreKeys / kPreChunk - 1; cp >= 0; --cp)
+                if (cp * kPreChunk < nk) {
+                    tmem_ld32(trow + cp * kPreChunk, v[0]);
+                    tmem_ld32(trow + cp * kPreChunk + 32, v[1]);
+                    tmem_wait_ld();
 #pragma unroll
-                for (int i = 0; i < 64; ++i) mx[i & 3] = fmaxf(mx[i & 3], __uint_as_float(v[i >> 5][i & 31]));
-                const float cmax = fmaxf(fmaxf(mx[0], mx[1]), fmaxf(mx[2], mx[3])) * scale;
-                if (cmax > m_run + 8.f) {
-                    const float al = fast_exp2(m_run - cmax);  // 0 when nothing came before
-                    l_run *= al;
-                    rs *= al;
-                    if (t >= 1) {  // O holds earlier tiles
-                        uint32_t o[32];
+                    for (int i = 0; i < 64; ++i) mx[i & 3] = fmaxf(mx[i & 3], __uint_as_float(v[i >> 5][i & 31]));
+                }
+            const float cmax = fmaxf(fmaxf(mx[0], mx[1]), fmaxf(mx[2], mx[3])) * scale;
+            if (cmax > m_run + 8.f) {
+                const float al = fast_exp2(m_run - cmax);  // 0 when nothing came before
+                l_run *= al;
+                if (t >= 1) {  // O holds earlier tiles
+                    uint32_t o[32];
 #pragma unroll
-                        for (int cb = 0; cb < D / 32; ++cb) {
-                            tmem_ld32(trow + O_COL + cb * 32, o);
-                            tmem_wait_ld();
-#pragma unroll
-                            for (int i = 0; i < 32; ++i) o[i] = __float_as_uint(__uint_as_float(o[i]) * al);
-                            tmem_st32(trow + O_COL + cb * 32, o);
-                        }
-                    }
-                    for (int cq = 0; cq < cp; ++cq) {  // this tile's earlier P words
-                        uint32_t w[32];
-                        tmem_ld32(trow + cq * 32, w);
+                    for (int cb = 0; cb < D / 32; ++cb) {
+                        tmem_ld32(trow + O_COL + cb * 32, o);
                         tmem_wait_ld();
 #pragma unroll
-                        for (int i = 0; i < 32; ++i)
-                            w[i] = pack_bf16(__uint_as_float(w[i] << 16) * al, __uint_as_float(w[i] & 0xFFFF0000u) * al);
-                        tmem_st32(trow + cq * 32, w);
+                        for (int i = 0; i < 32; ++i) o[i] = __float_as_uint(__uint_as_float(o[i]) * al);
+                        tmem_st32(trow + O_COL + cb * 32, o);
                     }
-                    m_run = cmax;
                 }
-                uint32_t w[32];
-                float r4[4] = {0.f, 0.f, 0.f, 0.f};
-#pragma unroll
-                for (int i = 0; i < 64; i += 2) {
-                    const float p0 = fast_exp2(fmaf(__uint_as_float(v[i >> 5][i & 31]), scale, -m_run));
-                    const float p1 = fast_exp2(fmaf(__uint_as_float(v[i >> 5][(i + 1) & 31]), scale, -m_run));
-                    r4[(i >> 1) & 3] += p0 + p1;
-                    w[i / 2] = pack_bf16(p0, p1);
-                }
-                rs += (r4[0] + r4[1]) + (r4[2] + r4[3]);
-                tmem_st32(trow + cp * 32, w);
+                m_run = cmax;
             }
-            l_run += rs;
-            tmem_wait_st();
-            tc_fence_before();
-            mbar_arrive(p_full(a));
+            // p = 2^(s * scale - m_ref) as bf16 pairs over the first columns
+            // of S (the A operand of P.V), one 64-key half at a time: the MMA
+            // thread starts on the first while the second is computed
+#pragma unroll
+            for (int cp = 0; cp < kPreKeys / kPreChunk; ++cp) {
+                if (cp * kPreChunk < nk) {
+                    if (cp > 0) {  // the first half's scores are still in v
+                        tmem_ld32(trow + cp * kPreChunk, v[0]);
+                        tmem_ld32(trow + cp * kPreChunk + 32, v[1]);
+                        tmem_wait_ld();
+                    }
+                    uint32_t w[32];
+                    float r4[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+                    for (int i = 0; i < 64; i += 2) {
+                        const uint32_t(&x)[32] = v[i >> 5];
+                        const float p0 = fast_exp2(fmaf(__uint_as_float(x[i & 31]), scale, -m_run));
+                        const float p1 = fast_exp2(fmaf(__uint_as_float(x[(i + 1) & 31]), scale, -m_run));
+                        r4[(i >> 1) & 3] += p0 + p1;
+                        w[i / 2] = pack_bf16(p0, p1);
+                    }
+                    l_run += (r4[0] + r4[1]) + (r4[2] + r4[3]);
+                    tmem_st32(trow + cp * 32, w);
+                    tmem_wait_st();
+                    tc_fence_before();
+                }
+                mbar_arrive(p_full(a, cp));
+            }
         }
         // ---- this CTA's record per (sharer, KV head) ----
         wait_phase(o_done(a), (uint32_t)(nt - 1) & 1u, c.err, dead);

@@ -476,7 +476,7 @@ namespace {
 constexpr double kSuffixGuess = 512;         // tokens of a sequence after its prefix
 constexpr double kStreamBytesPerUs = 6.5e6;  // of the decode kernel
 constexpr double kSplitUs = 10;              // a prefix CTA's start and end
-constexpr double kKeyTileUs = 2.7;           // its 128-key tile, beside the decode kernel
+constexpr double kKeyTileUs = 2;             // its 128-key tile, beside the decode kernel
 
 struct CascadePlan {
     const kv_prefix_group *groups;
@@ -611,6 +611,7 @@ int attn_call(kv_pool *p, int layout, const uint16_t *q, const uint16_t *k_new, 
     if (!workspace || ws_bytes < need || ((uintptr_t)workspace & 255u)) return KV_ERR_WORKSPACE;
     uint8_t *ws = reinterpret_cast<uint8_t *>(workspace);
     c->q = q;
+    c->pool = a.pool;
     c->table = dev_table;
     c->err = p->desc.device_error;
     c->ws_pre = reinterpret_cast<float *>(ws + pre_off);
