@@ -112,6 +112,9 @@ constexpr int kMinPartTokens = 64;
 // Below this many units a warp (by the table's width) a warp may have a single
 // unit and the CTAs merge in every mode.
 constexpr int kMergeUnits = 8;
+// Whose records a decode grid leaves, and how the combine finds a run's: each
+// warp's and each CTA's (MERGE) by run, or CTAs' by part (see attn_run).
+enum { kRecWarps = 0, kRecCtas = 1, kRecCtasByPart = 2 };
 constexpr uint32_t kHalfBytes = kTile * 128;      // one 64-column box: 16 rows x 128 B
 constexpr uint64_t kWaitLimitNs = 2000000000ull;  // bounded mbarrier waits: 2 s
 
@@ -142,7 +145,9 @@ struct AttnArgs {
     const int32_t *ctx_lens;
     int32_t *err;
     float *ws_part;
-    int2 *ws_run;            // per run: the parts of its records, [x, y); y = x if it has none
+    int2 *ws_run;            // per run: the parts of its records, [x, y); y = x if it has none.
+                             // kRecCtasByPart: per part, the run that starts in it and goes on
+                             // (x), and the one that ends in it and started earlier (y); or -1
     int64_t rows_per_page;   // page_bytes / (d * 2)
     int64_t pool_pages;
     int32_t pages_per_block;
@@ -867,10 +872,11 @@ __device__ __forceinline__ void issue_half(const CUtensorMap *tmap, const AttnAr
                                     policy, elected);
 }
 
-template <int D, int G, class Comp, bool MERGE>
+template <int D, int G, class Comp, int MODE>
 __global__ void __launch_bounds__(kThreads, Comp::kMinBlocks)
 paged_attn_kernel(const __grid_constant__ CUtensorMap tmap, const __grid_constant__ AttnArgs a)
 {
+    constexpr bool MERGE = MODE != kRecWarps, BY_PART = MODE == kRecCtasByPart;
     constexpr int HALVES = D / 64;
     constexpr int UNIT = kUnit<D>, SUB = kSub<D>;
     static_assert(HALVES == 1 || SUB == 1, "a unit's boxes follow each other in shared memory");
@@ -1006,7 +1012,8 @@ paged_attn_kernel(const __grid_constant__ CUtensorMap tmap, const __grid_constan
             // its output from the prefix records alone
             if (n == 0)
                 for (int i = 0; i < Hq * D; ++i) a.out[(int64_t)s * Hq * D + i] = 0;
-            for (int g = 0; g < Hkv; ++g) a.ws_run[(int64_t)s * Hkv + g] = make_int2(0, 0);
+            if (!BY_PART)
+                for (int g = 0; g < Hkv; ++g) a.ws_run[(int64_t)s * Hkv + g] = make_int2(0, 0);
         }
         __syncthreads();
     }
@@ -1022,10 +1029,14 @@ paged_attn_kernel(const __grid_constant__ CUtensorMap tmap, const __grid_constan
     const int32_t fine = a.min_units > 1 ? W / (NW * a.min_units) : (W + NW - 1) / NW;
     const int32_t NC = W > 0 ? min(max(fine, 1), a.P) : 0;
     const int32_t bid = (int32_t)blockIdx.x;
-    if (bid >= NC) {
+    auto no_part = [&]() {  // the CTA (without MERGE: this warp) has no units
+        if (BY_PART && tid == 0) {
+            make_ready();
+            a.ws_run[bid] = make_int2(-1, -1);
+        }
         if (chained) grid_dependency_wait();
-        return;
-    }
+    };
+    if (bid >= NC) return no_part();
     // first unit of CTA i: i * W / NC, with W = wq * NC + wr
     const int32_t wq = (int32_t)((uint32_t)W / (uint32_t)NC), wr = W - wq * NC;
     const float nc_inv = inv_of(NC);
@@ -1035,10 +1046,7 @@ paged_attn_kernel(const __grid_constant__ CUtensorMap tmap, const __grid_constan
     };
     const int32_t cu0 = cta_begin(bid), cu1 = cta_begin(bid + 1), nu = cu1 - cu0;  // this CTA's units
     const int32_t nw = min(NW, nu);  // warps with units (all but where W < NW)
-    if (!MERGE && warp >= nw) {  // no CTA-wide barrier below this point without MERGE
-        if (chained) grid_dependency_wait();
-        return;
-    }
+    if (!MERGE && warp >= nw) return no_part();  // no CTA-wide barrier below this point without MERGE
     // this warp's units
     const int32_t nq = (int32_t)((uint32_t)nu / (uint32_t)nw), nr = nu - nq * nw;
     const float nw_inv = inv_of(nw);
@@ -1091,6 +1099,7 @@ paged_attn_kernel(const __grid_constant__ CUtensorMap tmap, const __grid_constan
 
     bool dead = false;
     uint32_t consumed = 0;
+    int2 cut = make_int2(-1, -1);  // BY_PART: the part's entry, as far as this warp holds its ends
     int32_t u = u0;
     while (u < u1) {
         const int32_t n = seq_len(T, S, run.s), skip = seq_skip(T, S, run.s);
@@ -1178,6 +1187,8 @@ paged_attn_kernel(const __grid_constant__ CUtensorMap tmap, const __grid_constan
         // records begin and end
         const bool first = run.begin >= g0, last = run_end <= g1;
         const int end = split ? part + 1 : part;
+        if (BY_PART && pe == g1 && first && !last) cut.x = r;
+        if (BY_PART && u == g0 && last && !first) cut.y = r;
         uint16_t *orow = a.out + ((int64_t)run.s * Hq + (int64_t)run.g * G) * D;
         float *slot = a.ws_part + ((int64_t)r + part) * MF;
         // (MERGE) the part's share of the run; it may go on over several warps
@@ -1185,7 +1196,7 @@ paged_attn_kernel(const __grid_constant__ CUtensorMap tmap, const __grid_constan
         if (!MERGE || (u == lo && pe == hi)) {
             make_ready();
             comp.store(orow, slot, split, lane);
-            if (lane == 0) {
+            if (!BY_PART && lane == 0) {
                 if (first) a.ws_run[r].x = part;
                 if (last) a.ws_run[r].y = end;
             }
@@ -1200,6 +1211,11 @@ paged_attn_kernel(const __grid_constant__ CUtensorMap tmap, const __grid_constan
         }
         u = pe;
         run = next;
+    }
+    if (BY_PART && lane == 0 && u0 < u1) {
+        make_ready();
+        if (u1 == g1) a.ws_run[part].x = cut.x;
+        if (u0 == g0) a.ws_run[part].y = cut.y;
     }
     if constexpr (MERGE) {
         __syncthreads();
@@ -1240,8 +1256,8 @@ paged_attn_kernel(const __grid_constant__ CUtensorMap tmap, const __grid_constan
                     slot[G * D + G + h] = L;
                 }
             }
-            if (c == 0 && (ch.z & 1)) a.ws_run[ch.x].x = part;
-            if (c == 0 && (ch.z & 2)) a.ws_run[ch.x].y = part + ch.w;
+            if (c == 0 && (ch.z & 1) && !BY_PART) a.ws_run[ch.x].x = part;
+            if (c == 0 && (ch.z & 2) && !BY_PART) a.ws_run[ch.x].y = part + ch.w;
         }
     }
     if (chained) grid_dependency_wait();
@@ -1257,10 +1273,11 @@ paged_attn_kernel(const __grid_constant__ CUtensorMap tmap, const __grid_constan
 // by halves in a fixed order, so the result depends only on the run's shape.
 // (Merged one after another by the first group, 29 groups made a step of four
 // short sequences 3 µs longer: 15.4 µs against 12.4.)  Runs finished inside
-// the attention kernel return at once.
+// the attention kernel return at once; with very many runs (kRecCtasByPart) a
+// CTA per part takes the run that starts there and goes on.
 struct CombineArgs {
     uint16_t *out;
-    const int2 *ws_run;    // per run: the parts of its records, [x, y); y = x when not split
+    const int2 *ws_run;    // as in AttnArgs
     const float *ws_part;
     int32_t S;
     int32_t Hkv;
@@ -1327,7 +1344,27 @@ inline size_t combine_smem_bytes(int threads)
     return threads > CombineShape<D, G, CPT, CS>::NCT ? (size_t)threads * CPT * (2 * sizeof(float) + sizeof(float4)) : 0;
 }
 
-template <int D, int G, int CPT, int CS, bool WARPS>
+// The run of this CTA (-1: none) and the parts of its records, [at.x, at.y).
+template <int MODE>
+__device__ __forceinline__ int combine_run_of(const CombineArgs &c, int2 &at)
+{
+    const int b = blockIdx.x;
+    at = c.ws_run[b];
+    if constexpr (MODE != kRecCtasByPart) return b;
+    const int r = at.x;
+    at = make_int2(b, b);
+    // the run ends in the next part whose entry names it, 32 looked at at a
+    // time (the warps of a CTA all find the same)
+    const int ln = (int)threadIdx.x & 31, parts = gridDim.x;
+    if (r >= 0)
+        for (int q = b + 1; q < parts && at.y == b; q += 32) {
+            const unsigned hit = __ballot_sync(0xffffffffu, q + ln < parts && c.ws_run[q + ln].y == r);
+            if (hit) at.y = q + __ffs((int)hit);
+        }
+    return r;
+}
+
+template <int D, int G, int CPT, int CS, int MODE>
 __global__ void __launch_bounds__(CombineShape<D, G, CPT, CS>::MAX_THREADS, CombineShape<D, G, CPT, CS>::MIN_CTAS)
 combine_kernel(const __grid_constant__ CombineArgs c)
 {
@@ -1338,14 +1375,16 @@ combine_kernel(const __grid_constant__ CombineArgs c)
     static_assert(Sh::NC % CPT == 0 && NCT <= kCombineMaxThreads, "whole columns per thread");
     const int NG = (int)blockDim.x / NCT;  // groups of NCT threads
     extern __shared__ float4 s_dyn[];      // [CPT][blockDim] O, then M, then L (when NG > 1)
-    const int r = blockIdx.x;
     grid_dependency_wait();  // the attention grid's partials and run table
     // Release the next grid only now, when every grid before this one has
     // completed: a decode grid that follows without a wait of its own (step
     // overlap) relies on it, and until its own wait writes nothing that this
     // grid reads or writes.
     grid_launch_dependents();
-    const int2 info = c.ws_run[r];
+    int2 at;
+    const int r = combine_run_of<MODE>(c, at);
+    if (MODE == kRecCtasByPart && r < 0) return;  // no run starts in this part and goes on
+    const int2 info = at;
     const int s = r / c.Hkv, g = r % c.Hkv;
     const int npre = (c.skip != nullptr && c.skip[s] > 0) ? c.KS : 0;
     const int cnt = info.y - info.x + npre;
@@ -1374,7 +1413,7 @@ combine_kernel(const __grid_constant__ CombineArgs c)
     auto record = [&](int k) {
         return k < npre ? c.ws_pre + ((int64_t)k * (int)gridDim.x + r) * MF : base + (int64_t)(k - npre) * MF;
     };
-    if constexpr (!WARPS) {
+    if constexpr (MODE != kRecWarps) {
         for (int k0 = grp; k0 < cnt; k0 += NG * B) {
             float mv[B][CPT], lv[B][CPT];
             float4 ov[B][CPT];

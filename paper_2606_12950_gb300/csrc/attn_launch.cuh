@@ -47,28 +47,28 @@ int cached_occupancy(Fn fn, int threads, size_t smem, int *occ, OccCache &c)
 }
 
 // The combine over c's runs: `groups` thread groups a CTA, CS CTAs a run.
-template <int D, int G, int CPT, int CS, bool WARPS>
-int combine_launch(const CombineArgs &c, int groups, cudaLaunchConfig_t cfg)
+template <int D, int G, int CPT, int CS, int MODE>
+int combine_launch(const CombineArgs &c, int groups, cudaLaunchConfig_t cfg, int parts = 0)
 {
     const int threads = groups * CombineShape<D, G, CPT, CS>::NCT;
-    cfg.gridDim = dim3((unsigned)(c.S * c.Hkv), (unsigned)CS);
+    cfg.gridDim = dim3((unsigned)(MODE == kRecCtasByPart ? parts : c.S * c.Hkv), (unsigned)CS);
     cfg.blockDim = dim3((unsigned)threads);
     cfg.dynamicSmemBytes = combine_smem_bytes<D, G, CPT, CS>(threads);
-    if (cudaLaunchKernelEx(&cfg, combine_kernel<D, G, CPT, CS, WARPS>, c) != cudaSuccess) return KV_ERR_CUDA;
+    if (cudaLaunchKernelEx(&cfg, combine_kernel<D, G, CPT, CS, MODE>, c) != cudaSuccess) return KV_ERR_CUDA;
     kvp_note_stream(cfg.stream, true);
     return KV_OK;
 }
 
 // Few runs: each run's columns spread over CS CTAs (kSlicedCtas).
-template <int D, int G, bool WARPS>
+template <int D, int G, int MODE>
 int combine_run(const CombineArgs &c, double per_run, int sm_count, const cudaLaunchConfig_t &cfg)
 {
     const int runs = c.S * c.Hkv;
     if (8 * runs <= kSlicedCtas * sm_count)
-        return combine_launch<D, G, 1, 8, WARPS>(c, combine_groups<D, G, 8>(per_run), cfg);
+        return combine_launch<D, G, 1, 8, MODE>(c, combine_groups<D, G, 8>(per_run), cfg);
     if (4 * runs <= kSlicedCtas * sm_count)
-        return combine_launch<D, G, 1, 4, WARPS>(c, combine_groups<D, G, 4>(per_run), cfg);
-    return combine_launch<D, G, 1, 1, WARPS>(c, combine_groups<D, G, 1>(per_run), cfg);
+        return combine_launch<D, G, 1, 4, MODE>(c, combine_groups<D, G, 4>(per_run), cfg);
+    return combine_launch<D, G, 1, 1, MODE>(c, combine_groups<D, G, 1>(per_run), cfg);
 }
 
 // what: kLaunchQuery (only *P_out), kLaunchBoth (attention, then combine),
@@ -78,12 +78,14 @@ enum { kLaunchQuery = 0, kLaunchBoth = 1, kLaunchAttention = 2, kLaunchCombine =
 template <int D, int G, class Comp>
 int attn_run(const CUtensorMap *tmap, AttnArgs a, int P_req, int sm_count, cudaStream_t st, int what, int *P_out)
 {
-    auto fn = paged_attn_kernel<D, G, Comp, false>;
-    auto fn_merge = paged_attn_kernel<D, G, Comp, true>;
+    auto fn = paged_attn_kernel<D, G, Comp, kRecWarps>;
+    auto fn_merge = paged_attn_kernel<D, G, Comp, kRecCtas>;
+    auto fn_by_part = paged_attn_kernel<D, G, Comp, kRecCtasByPart>;
     static std::atomic<bool> attr_set{false};
     if (!attr_set.load()) {
         if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemMax) != cudaSuccess ||
-            cudaFuncSetAttribute(fn_merge, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemMax) != cudaSuccess)
+            cudaFuncSetAttribute(fn_merge, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemMax) != cudaSuccess ||
+            cudaFuncSetAttribute(fn_by_part, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemMax) != cudaSuccess)
             return KV_ERR_CUDA;
         attr_set.store(true);
     }
@@ -130,6 +132,19 @@ int attn_run(const CUtensorMap *tmap, AttnArgs a, int P_req, int sm_count, cudaS
             if (small) a.min_units = 1;
         }
     }
+    // At most one run per part starts there and goes on.  With several waves
+    // of runs (eight runs a part: two waves of 128-thread combine CTAs) the
+    // combine gets a CTA per part instead of one per run, most of which only
+    // had to find their run whole: three co-located models (6560, 1640 and 816
+    // runs) 266.4 -> 261.0 us, 1024 long contexts (8192) 691.4 -> 686.6, 1000
+    // sequences of 400 tokens (8000) 263.5 -> 257.2.  With 960 and 1024 runs the
+    // look for the run's end costs more than it saves: 92.8 -> 93.5 and 69.0 ->
+    // 69.9.
+    // (Never with runs few enough for column slices: the order of the merge
+    // would differ from the overlapped form's.)
+    const int64_t n_runs = (int64_t)a.S * a.Hkv;
+    const bool by_part = merge && a.skip == nullptr && n_runs >= 8 * (int64_t)P && 4 * n_runs > (int64_t)kSlicedCtas * sm_count;
+    if (by_part) fn = fn_by_part;
     // both kernels are programmatic dependents of what precedes them in the
     // stream: they may be scheduled early and wait on the device
     // (griddepcontrol.wait) for the previous grid to complete
@@ -159,10 +174,11 @@ int attn_run(const CUtensorMap *tmap, AttnArgs a, int P_req, int sm_count, cudaS
         // one group in shared-prefix mode: two columns a thread, so that
         // every member run fits in one wave
         if (a.skip != nullptr && combine_groups<D, G, 1>(per_run) == 1)
-            return combine_launch<D, G, 2, 1, false>(c, 1, ccfg);
+            return combine_launch<D, G, 2, 1, kRecCtas>(c, 1, ccfg);
     }
-    return merge || a.skip != nullptr ? combine_run<D, G, false>(c, per_run, sm_count, ccfg)
-                                      : combine_run<D, G, true>(c, per_run, sm_count, ccfg);
+    if (by_part) return combine_launch<D, G, 1, 1, kRecCtasByPart>(c, combine_groups<D, G, 1>(per_run), ccfg, P);
+    return merge || a.skip != nullptr ? combine_run<D, G, kRecCtas>(c, per_run, sm_count, ccfg)
+                                      : combine_run<D, G, kRecWarps>(c, per_run, sm_count, ccfg);
 }
 
 // Shared-prefix kernel: with launch = false only reports the CTAs that fit

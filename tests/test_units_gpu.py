@@ -208,3 +208,38 @@ def test_records_per_warp_and_per_cta_give_the_same_bits(G, Hkv, d, variant, len
         assert np.array_equal(alone, db.out_bits()), splits
     _check(db.out_f64(), oracle.batch_attention(b, pool=oracle.batch_append(b)), (G, Hkv, d))
     assert pool.error() == 0
+
+
+@pytest.mark.parametrize("G,Hkv,d", [(1, 8, 128), (4, 4, 64)])
+@pytest.mark.parametrize("splits", [1, 2, 3, 16, 40, 0])
+def test_combine_by_part(splits, G, Hkv, d):
+    """Many more runs than parts (with the splits given; at 0, 2560 runs on 304
+    CTAs): the combine has a CTA per part, for the run that starts there.  Runs
+    inside a part, over two and over many, empty sequences, and parts without
+    units; against the oracle, and bit for bit against the same call overlapping
+    another's combine, which has a CTA per run."""
+    from paper_2606_12950_gb300.runner import DeviceBatch, DevicePool
+
+    S = 2560 // Hkv if splits == 0 else 200 // Hkv * 2
+    lens = [7 + 29 * s % 150 for s in range(S)]
+    lens[3], lens[S // 2], lens[S - 1] = 6000, 900, 2000
+    width = None
+    if splits == 40:  # one unit a run, so most of the CTAs have none
+        lens, width = [3 + s % 12 for s in range(400 // Hkv)], 4096
+    b = W.make_batch(7600 + G + d, lens, Hq=G * Hkv, Hkv=Hkv, d=d, bs=16, extra_blocks=3, max_blocks=width)
+    post = b.ctx_lens.copy()
+    post[[0, 5, 6]] = 0  # empty
+    b.ctx_lens = post
+    pool = DevicePool(b.n_pages, b.page_elems * 2, b.bs, [(b.Hkv, b.d)])
+    pool.upload(b.pool)
+    db = DeviceBatch(pool, 0, b, splits)
+    db.attend()
+    torch.cuda.synchronize()
+    alone = db.out_bits()
+    _check(db.out_f64(), oracle.batch_attention(b, pool=b.pool), (splits, G))
+    pool.set_step_overlap(True)
+    for _ in range(3):
+        db.attend()
+    torch.cuda.synchronize()
+    assert np.array_equal(alone, db.out_bits())
+    assert pool.error() == 0
