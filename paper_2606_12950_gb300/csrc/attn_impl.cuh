@@ -1353,12 +1353,15 @@ __device__ __forceinline__ int combine_run_of(const CombineArgs &c, int2 &at)
     if constexpr (MODE != kRecCtasByPart) return b;
     const int r = at.x;
     at = make_int2(b, b);
-    // the run ends in the next part whose entry names it, 32 looked at at a
-    // time (the warps of a CTA all find the same)
+    // The run ends in the next part whose entry names it.  Each warp looks for
+    // itself, a part a lane; a CTA's threads need not be whole warps (80 of
+    // them with five query heads of 64), so the last warp may have fewer lanes.
     const int ln = (int)threadIdx.x & 31, parts = gridDim.x;
+    const int lanes = min(32, (int)blockDim.x - ((int)threadIdx.x & ~31));
+    const unsigned mask = 0xffffffffu >> (32 - lanes);
     if (r >= 0)
-        for (int q = b + 1; q < parts && at.y == b; q += 32) {
-            const unsigned hit = __ballot_sync(0xffffffffu, q + ln < parts && c.ws_run[q + ln].y == r);
+        for (int q = b + 1; q < parts && at.y == b; q += lanes) {
+            const unsigned hit = __ballot_sync(mask, q + ln < parts && c.ws_run[q + ln].y == r);
             if (hit) at.y = q + __ffs((int)hit);
         }
     return r;

@@ -243,3 +243,55 @@ def test_combine_by_part(splits, G, Hkv, d):
     torch.cuda.synchronize()
     assert np.array_equal(alone, db.out_bits())
     assert pool.error() == 0
+
+
+def _long_run_units(span, short_runs, P, min_units, before=5):
+    """Units of a run that starts after `before` one-unit runs and ends `span`
+    parts after the one it starts in, by the kernel's cut: W units in NC equal
+    ranges, NC = min(max(W // (6 * min_units), 1), P)."""
+    for n in range(2, 1 << 16):
+        w = short_runs + n
+        nc = min(max(w // (6 * min_units), 1), P)
+        begin = np.arange(nc + 1) * w // nc
+        first, last = np.searchsorted(begin, [before, before + n - 1], "right") - 1
+        if last - first == span:
+            return n
+    raise AssertionError(span)
+
+
+@pytest.mark.parametrize("d", [64, 128])
+@pytest.mark.parametrize("G", [1, 2, 4, 5, 8])
+def test_combine_by_part_finds_the_end_of_a_run(G, d):
+    """A combine CTA per part, and a run that ends 1 to 49 parts after the one it
+    starts in: the look for its end takes one pass or two, by warps of 32 lanes
+    and, with 80 threads a CTA (G = 5 at d = 64), of 16.  Every output is
+    written (NaN before the call), against the oracle, and bit for bit as the
+    overlapped form, which has a combine CTA per run.
+
+    Contexts of a token or a few have outputs as large as the values, so the bar
+    is the roundings' bound: a weight to bf16, 2^-9 of it, so 2^-9 max|v| of the
+    output; the output itself, 2^-9 |out|; fp32 sums, below 2^-6 of those."""
+    from paper_2606_12950_gb300.runner import DeviceBatch, DevicePool
+
+    P, S, unit = 60, 600, 32 if d == 64 else 16
+    for span in (1, 15, 16, 17, 31, 32, 33, 49):
+        lens = [s % 15 for s in range(S)]
+        lens[5] = _long_run_units(span, S - 1, P, 64 // unit) * unit - 3
+        b = W.make_batch(7800 + span + G, lens, Hq=G, Hkv=1, d=d, bs=16, extra_blocks=3)
+        pool = DevicePool(b.n_pages, b.page_elems * 2, b.bs, [(1, d)])
+        pool.upload(b.pool)
+        db = DeviceBatch(pool, 0, b, P)
+        db.out.fill_(float("nan"))
+        db.attend()
+        torch.cuda.synchronize()
+        alone = db.out_bits()
+        ref = oracle.batch_attention(b, pool=b.pool)
+        vmax = np.abs(W.bf16_bits_to_f64(b.pool)).max()
+        assert np.all(np.abs(db.out_f64() - ref) <= (2.0 ** -9 + 2.0 ** -15) * (vmax + np.abs(ref))), (span, G, d)
+        pool.set_step_overlap(True)
+        db.attend()
+        db.out.fill_(float("nan"))
+        db.attend()
+        torch.cuda.synchronize()
+        assert np.array_equal(alone, db.out_bits()), (span, G, d)
+        assert pool.error() == 0
