@@ -82,10 +82,13 @@ namespace {
 // Append: the decode step writes the new token's K and V before attending
 // (§II).  One thread per 16-byte chunk of a (sequence, KV head, K|V) row; 16
 // consecutive threads write one 256-byte row (d = 128), so stores coalesce.
-__global__ void append_kernel(uint8_t *__restrict__ pool, const uint4 *__restrict__ k_new,
-                              const uint4 *__restrict__ v_new, const int32_t *__restrict__ table,
-                              const int32_t *__restrict__ ctx_lens, int32_t *err, int S, int Hkv, int D, int bs,
-                              int max_blocks, int64_t page_bytes, int64_t n_pages, int32_t pages_per_block)
+// No __restrict__: the kernel may be resident while the grid before it (the
+// table sync, say) still writes the lengths, the table or the rows, and a
+// const __restrict__ pointer may be read through the non-coherent path, which
+// the wait below does not order.
+__global__ void append_kernel(uint8_t *pool, const uint4 *k_new, const uint4 *v_new, const int32_t *table,
+                              const int32_t *ctx_lens, int32_t *err, int S, int Hkv, int D, int bs, int max_blocks,
+                              int64_t page_bytes, int64_t n_pages, int32_t pages_per_block)
 {
     // Launched as a programmatic dependent, like the kernels around it: the
     // grids before may still read what is written here until this wait, and

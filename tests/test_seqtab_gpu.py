@@ -115,3 +115,52 @@ def test_fused_sync_gives_the_bits_of_sync_then_attention(S):
     for pool, t, _ in sides:
         t.close()
         pool.close()
+
+
+@pytest.mark.parametrize("S", [4, 200])
+def test_append_after_a_sync_sees_this_steps_lengths(S):
+    """kv_seqtab_sync, kv_append, paged_decode_attn, step after step with nothing
+    between them: the append, resident before the sync kernel has written this
+    step's lengths and table, puts each row where the fused call puts it.  Every
+    step's output and the pool bit for bit, with a row of its own each step."""
+    from paper_2606_12950_gb300.runner import DevicePool, DeviceSteps
+
+    Hq, Hkv, d, bs, max_blocks, steps = 8, 2, 128, 16, 8, 60
+    n_pages, page_elems = S * max_blocks, 2 * Hkv * bs * d
+    rng = np.random.default_rng(S)
+
+    def bits(*shape):
+        return (rng.standard_normal(shape).astype(np.float32).view(np.uint32) >> 16).astype(np.uint16)
+
+    host_pool, q, kn, vn = bits(n_pages * page_elems), bits(S, Hq, d), bits(S, Hkv, d), bits(S, Hkv, d)
+    start = rng.integers(1, 2 * bs, S)
+    outs, pools = [], []
+    for fused in (False, True):
+        pool = DevicePool(n_pages, page_elems * 2, bs, [(Hkv, d)], shuffle_seed=5)
+        pool.upload(host_pool)
+        t = K.SeqTab(pool.handle, 0, S, max_blocks)
+        buf = DeviceSteps(pool, 0, S, S, Hq, Hkv, d, max_blocks, d ** -0.5, q, kn, vn)
+        k0, v0 = buf.k_new.clone(), buf.v_new.clone()
+        for s in range(S):
+            t.reserve(s, int(start[s]))
+            t.set_len(s, int(start[s]))
+        seen = []
+        for step in range(steps):
+            buf.k_new.copy_(k0 * (step + 1))
+            buf.v_new.copy_(v0 * (step + 1))
+            t.advance(list(range(S)))
+            if fused:
+                buf.sync_append_attend(t)
+            else:
+                buf.sync(t)
+                buf.append()
+                buf.attend()
+            seen.append(buf.out.clone())
+        torch.cuda.synchronize()
+        assert pool.error() == 0
+        outs.append(torch.stack(seen).view(torch.int16).cpu().numpy())
+        pools.append(pool.download())
+        t.close()
+        pool.close()
+    assert np.array_equal(outs[0], outs[1])
+    assert np.array_equal(pools[0], pools[1])
