@@ -1502,11 +1502,14 @@ combine_kernel(const __grid_constant__ CombineArgs c)
 // host helpers ---------------------------------------------------------------
 constexpr int kRowsCap = 2048;
 
+// shared memory of a decode CTA; with boxes = 1, what it would be with a unit
+// of a box (the S that a call may have, see attn_run)
 template <int D, int G>
-inline size_t attn_smem_bytes(int S, int rows_cap, int nwarps, bool merge)
+inline size_t attn_smem_bytes(int S, int rows_cap, int nwarps, bool merge, int boxes = kSub<D>)
 {
-    const size_t stage = 2ull * (D / 64) * kSub<D> * kHalfBytes;
-    const size_t bufs = (size_t)G * D * 2 + 2 * D * 2 + (merge ? merge_floats<D, G>() * 4 + 16 : 0);  // per warp: q rows, new K/V rows; a record, its chain
+    const size_t stage = 2ull * (D / 64) * boxes * kHalfBytes;
+    // per warp: q rows, new K/V rows; a record, its chain
+    const size_t bufs = (size_t)G * D * 2 + 2 * D * 2 + (merge ? merge_floats<D, G>() * 4 + 16 : 0);
     return 1024 + (size_t)nwarps * (kStages * stage + bufs) + (2 * nwarps * kStages) * 8 + 64 + (size_t)(3 * S + 1) * 4 +
            (size_t)rows_cap * 4;
 }

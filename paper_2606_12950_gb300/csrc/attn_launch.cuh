@@ -90,9 +90,16 @@ int attn_run(const CUtensorMap *tmap, AttnArgs a, int P_req, int sm_count, cudaS
         attr_set.store(true);
     }
     // six warps a CTA, eight beside the shared-prefix kernel (kPlainWarps)
-    a.nwarps = a.skip != nullptr ? kWarps : kPlainWarps;
+    const int most_warps = a.skip != nullptr ? kWarps : kPlainWarps;
+    // S too large for the per-CTA sequence index beside a box of K and of V a
+    // warp (14109 sequences at d = 128, 16349 at d = 64, one query head a KV
+    // head).  A unit of two boxes (d = 64) does not lower that limit: past
+    // 14301 sequences fewer warps take their stages from what the index leaves,
+    // three at the least.  There a CTA is alone on its SM either way.
+    if (attn_smem_bytes<D, G>(a.S, kRowsCap, most_warps, false, 1) > kSmemMax) return KV_ERR_INVALID_ARG;
+    a.nwarps = most_warps;
+    while (attn_smem_bytes<D, G>(a.S, kRowsCap, a.nwarps, false) > kSmemMax) --a.nwarps;
     size_t smem = attn_smem_bytes<D, G>(a.S, kRowsCap, a.nwarps, false);
-    if (smem > kSmemMax) return KV_ERR_INVALID_ARG;  // S too large for the per-CTA sequence index
     int occ = 0;
     static OccCache occ_cache;
     if (cached_occupancy(fn, a.nwarps * 32, smem, &occ, occ_cache) != KV_OK) return KV_ERR_CUDA;
@@ -117,7 +124,9 @@ int attn_run(const CUtensorMap *tmap, AttnArgs a, int P_req, int sm_count, cudaS
     const bool small = most_units < (int64_t)kMergeUnits * P * a.nwarps;
     bool merge = false;
     a.min_units = kMinPartTokens / kUnit<D>;
-    if (small || (a.chain != 3 && a.skip == nullptr)) {
+    // (with fewer warps the combine, which merges kPlainWarps records at a time,
+    // would not give a CTA's bits)
+    if (a.nwarps == most_warps && (small || (a.chain != 3 && a.skip == nullptr))) {
         const size_t smem_merge = attn_smem_bytes<D, G>(a.S, kRowsCap, a.nwarps, true);
         int occ_merge = 0;
         static OccCache merge_cache;

@@ -295,3 +295,37 @@ def test_combine_by_part_finds_the_end_of_a_run(G, d):
         torch.cuda.synchronize()
         assert np.array_equal(alone, db.out_bits()), (span, G, d)
         assert pool.error() == 0
+
+
+@pytest.mark.parametrize("G,d,S", [(1, 64, 14302), (1, 64, 15100), (1, 64, 16349), (8, 64, 15901), (4, 128, 13725)])
+def test_the_most_sequences_a_call_takes(G, d, S):
+    """S up to what the sequence index of a CTA leaves room for beside a 16-token
+    box of K and of V for each of six warps, whatever a unit holds: the last S
+    of each form is that limit, and one more is refused."""
+    from paper_2606_12950_gb300 import kvpool as K
+    from paper_2606_12950_gb300.runner import DeviceBatch, DevicePool
+
+    lens = [s % 19 for s in range(S)]
+    lens[7], lens[S - 3] = 3000, 700
+    b = W.make_batch(7900 + G, lens, Hq=G, Hkv=1, d=d, bs=16, extra_blocks=3)
+    pool = DevicePool(b.n_pages, b.page_elems * 2, b.bs, [(1, d)])
+    pool.upload(b.pool)
+    db = DeviceBatch(pool, 0, b)
+    db.append_attend()
+    torch.cuda.synchronize()
+    alone = db.out_bits()
+    ref_pool = oracle.batch_append(b)
+    assert np.array_equal(pool.download(), ref_pool)
+    ref = oracle.batch_attention(b, pool=ref_pool)
+    # contexts of a token or a few: the bound of the roundings (see above)
+    vmax = np.abs(W.bf16_bits_to_f64(ref_pool)).max()
+    assert np.all(np.abs(db.out_f64() - ref) <= (2.0 ** -9 + 2.0 ** -15) * (vmax + np.abs(ref)))
+    pool.set_step_overlap(True)
+    for _ in range(3):
+        db.append_attend()
+    torch.cuda.synchronize()
+    assert np.array_equal(alone, db.out_bits())
+    assert pool.error() == 0
+    if S in (16349, 15901, 13725):
+        with pytest.raises(K.KVError):
+            K.kv_workspace_bytes(pool.handle, 0, S + 1, G, b.max_blocks, 0)
