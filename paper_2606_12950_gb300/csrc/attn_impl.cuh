@@ -115,6 +115,12 @@ constexpr int kMergeUnits = 8;
 // Whose records a decode grid leaves, and how the combine finds a run's: each
 // warp's and each CTA's (MERGE) by run, or CTAs' by part (see attn_run).
 enum { kRecWarps = 0, kRecCtas = 1, kRecCtasByPart = 2 };
+// Where a state's running maximum starts.  Finite, so that a token whose score
+// is -inf gets weight 0 also before any other (2^(-inf - m), not 2^NaN), and so
+// that no record of a part has m = -inf, which stands for "no record" in the
+// merges: a part whose scores are all NaN leaves this m with l = NaN, and the
+// output is NaN, however the run was cut.
+constexpr float kMaxStart = -3.402823466e+38f;  // the lowest float
 constexpr uint32_t kHalfBytes = kTile * 128;      // one 64-column box: 16 rows x 128 B
 constexpr uint64_t kWaitLimitNs = 2000000000ull;  // bounded mbarrier waits: 2 s
 
@@ -279,7 +285,7 @@ struct FmaCompute {
             }
 #pragma unroll
             for (int e = 0; e < EPL / 2; ++e) o[h][e] = make_float2(0.f, 0.f);
-            m[h] = -INFINITY;
+            m[h] = kMaxStart;
             l[h] = 0.f;
         }
     }
@@ -459,7 +465,7 @@ struct MmaCompute {
 #pragma unroll
             for (int e = 0; e < 4; ++e) acc[kk][e] = 0.f;
         }
-        m[0] = m[1] = -INFINITY;
+        m[0] = m[1] = kMaxStart;
         l[0] = l[1] = 0.f;
     }
 

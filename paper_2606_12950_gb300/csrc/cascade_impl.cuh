@@ -384,7 +384,7 @@ cascade_prefix_kernel(const __grid_constant__ CUtensorMap tmap, const __grid_con
         const int a = qa_tile;
         const uint32_t trow = tbase + a * kPreTmemCols + ((uint32_t)((warp % 4) * 32) << 16);
         const float scale = c.qk_scale;
-        float m_run = -INFINITY, l_run = 0.f;
+        float m_run = kMaxStart, l_run = 0.f;
         for (int t = 0; t < nt; ++t) {
             const int nk = tile_keys(t);  // 128 or 64
             // S_a(t) complete: so is every earlier MMA of the tile, in

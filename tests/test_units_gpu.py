@@ -329,3 +329,104 @@ def test_the_most_sequences_a_call_takes(G, d, S):
     if S in (16349, 15901, 13725):
         with pytest.raises(K.KVError):
             K.kv_workspace_bytes(pool.handle, 0, S + 1, G, b.max_blocks, 0)
+
+
+def _exact(b, pool, s):
+    """Sequence s of batch b in 64 bits (NaN and infinities as IEEE has them)."""
+    n = int(b.ctx_lens[s])
+    kv = W.bf16_bits_to_f64(pool).reshape(-1, 2, b.Hkv, b.bs, b.d)[b.table[s, : -(-n // b.bs)]]
+    k, v = (kv[:, i].transpose(1, 0, 2, 3).reshape(b.Hkv, -1, b.d)[:, :n] for i in (0, 1))
+    q = W.bf16_bits_to_f64(b.q[s]).reshape(b.Hkv, b.G, b.d)
+    with np.errstate(all="ignore"):
+        x = q @ k.transpose(0, 2, 1) * b.scale
+        w = np.exp(x - x.max(-1, keepdims=True))
+        return ((w / w.sum(-1, keepdims=True)) @ v).reshape(b.Hq, b.d)
+
+
+@pytest.mark.parametrize("path", ["small", "per_cta", "per_warp", "cuda_cores", "prefix"])
+@pytest.mark.parametrize("d", [64, 128])
+def test_nan_and_infinite_scores(d, path):
+    """A token whose score is NaN makes its sequence's output NaN, and one whose
+    score is -inf has no weight, wherever the token is: alone in the run's last
+    unit (the new token), the first token, all of the first units, one in the
+    middle.  In every form of the records; the other sequences are as ever."""
+    from paper_2606_12950_gb300 import kvpool as K
+    from paper_2606_12950_gb300.runner import DeviceBatch, DevicePool
+
+    pre = [448, 448, 1000, 1000, 2048, 2048, 700, 330, 5000]
+    b = W.make_batch(8000 + d, pre, Hq=8, Hkv=2, d=d, bs=16, extra_blocks=3)
+    groups = [([4, 5, 6], 256)]
+    if path == "prefix":
+        W.share_prefix(b, groups)
+    one, nan, ninf = 0x3F80, 0x7FC0, 0xFF80
+    b.q[:, :, 0] = one
+    rows = b.pool.reshape(b.n_pages, 2, b.Hkv, b.bs, b.d)
+
+    def set_k(s, pos, bits):
+        rows[b.table[s, pos // b.bs], 0, 1, pos % b.bs, 0] = bits  # KV head 1
+
+    b.k_new[0, 1, 0] = nan      # the new token, the only one of its unit
+    b.k_new[1, 1, 0] = ninf
+    set_k(2, 0, nan)
+    for pos in range(64):       # whole units without a score
+        set_k(3, pos, ninf)
+    if path == "prefix":        # in the shared prefix: a NaN that all members see
+        set_k(4, 130, nan)
+        nan_seqs = [0, 2, 4, 5, 6]
+    else:
+        set_k(4, 1030, nan)
+        for pos in range(512):
+            set_k(5, pos, ninf)
+        nan_seqs = [0, 2, 4]
+    if path in ("per_cta", "per_warp", "cuda_cores"):  # a table too wide for the small batches' rule
+        wide = np.full((b.S, 16384), -1, np.int32)
+        wide[:, : b.max_blocks] = b.table
+        b.table, b.max_blocks = wide, 16384
+    pool = DevicePool(b.n_pages, b.page_elems * 2, b.bs, [(b.Hkv, b.d)])
+    pool.upload(b.pool)
+    pool.set_variant(1 if path == "cuda_cores" else 2)
+    db = DeviceBatch(pool, 0, b)
+    if path == "prefix":
+        db.cascade(K.PrefixPlan(groups))
+    else:
+        db.append_attend()
+    if path == "per_warp":
+        pool.set_step_overlap(True)
+        for _ in range(2):
+            db.append_attend()
+    torch.cuda.synchronize()
+    got, ref_pool = db.out_f64().reshape(b.S, b.Hq, d), oracle.batch_append(b)
+    for s in range(b.S):
+        ref = _exact(b, ref_pool, s)
+        if s in nan_seqs:
+            assert np.isnan(got[s, 4:]).all() and np.isnan(ref[4:]).all(), s
+            _check(got[s, :4], ref[:4], (s, path))
+        else:
+            _check(got[s], ref, (s, path))
+    assert pool.error() == 0
+
+
+@pytest.mark.parametrize("d", [64, 128])
+def test_shared_prefix_whose_first_keys_have_no_weight(d):
+    """-inf scores in the first 192 keys of a shared prefix: more than the first
+    128-key tile of the prefix kernel."""
+    from paper_2606_12950_gb300 import kvpool as K
+    from paper_2606_12950_gb300.runner import DeviceBatch, DevicePool
+
+    groups = [([0, 1, 2], 2048)]
+    b = W.make_batch(8100 + d, [2048, 2100, 2500, 40], Hq=8, Hkv=2, d=d, bs=16, extra_blocks=3)
+    W.share_prefix(b, groups)
+    b.q[:, :, 0] = 0x3F80
+    rows = b.pool.reshape(b.n_pages, 2, b.Hkv, b.bs, b.d)
+    for pos in range(192):
+        rows[b.table[0, pos // b.bs], 0, :, pos % b.bs, 0] = 0xFF80
+    pool = DevicePool(b.n_pages, b.page_elems * 2, b.bs, [(b.Hkv, b.d)])
+    pool.upload(b.pool)
+    db = DeviceBatch(pool, 0, b)
+    db.cascade(K.PrefixPlan(groups))
+    torch.cuda.synchronize()
+    ref_pool = oracle.batch_append(b)
+    got = db.out_f64().reshape(b.S, b.Hq, d)
+    for s in range(b.S):
+        _check(got[s], _exact(b, ref_pool, s), s)
+    assert pool.error() == 0
