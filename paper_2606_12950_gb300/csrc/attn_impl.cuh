@@ -165,7 +165,8 @@ struct AttnArgs {
     int32_t rows_cap;        // boxes whose pool rows are resolved up front
     int32_t P;               // CTAs
     int32_t nwarps;          // warps per CTA (<= kWarps)
-    int32_t min_units;       // least units of a warp (but in a CTA with fewer units than warps)
+    int32_t min_units;       // least units of a warp (but in a CTA with fewer units than warps);
+                             // to attn_run: in a small batch, 0 = 1
     float qk_scale;          // scale * log2(e)
     // shared-prefix (cascade) mode: tokens of each sequence's prefix handled
     // by the prefix kernel ([S], multiples of 16; null = none), its records
@@ -176,16 +177,16 @@ struct AttnArgs {
     // place in a chain of grids: 0 alone (release the next grid, then wait
     // for the one before); 1 first of a chain (wait, then release: the next
     // grid relies on this wait); 2 chained (release, no wait at the start,
-    // a wait at every exit: see the kernel); 3 right after a split-K combine
+    // a wait at the exit: see the kernel); 3 right after a split-K combine
     // of this library, which released this grid only after its own wait, so
     // every grid before that combine has completed (release, no wait at the
     // start, a wait before the first write of the output or the workspace,
-    // which the combine still uses, and at every exit); 4 beside the
+    // which the combine still uses, and at the exit); 4 beside the
     // shared-prefix kernel while the previous step's shared-prefix combine
     // finishes (release, no wait at the start; the plan kernel's two flags,
     // below, stand in for the waits: the first before anything the plan
     // kernel writes is read, the second before the first write of the output
-    // or the workspace; a wait for the prefix grid at every exit)
+    // or the workspace; a wait for the prefix grid at the exit)
     int32_t chain;
     // chain 4: the plan kernel sets flags[0] = epoch once the plan, the
     // skips and the table sync are written, and flags[1] = epoch once every
@@ -923,8 +924,9 @@ paged_attn_kernel(const __grid_constant__ CUtensorMap tmap, const __grid_constan
     // released it only after its own wait had seen every earlier grid
     // complete; it does not wait for that grid here, so the two run side by
     // side (the later one's CTAs take the SMs the earlier one frees), and
-    // waits for it at every exit (`chained`), so that a combine after it
-    // sees every chained grid's records.  Data from earlier grids is then
+    // waits for it at the exit (`chained`; all but CTAs without units, and
+    // CTA 0 always), so that a combine after it sees every chained grid's
+    // records.  Data from earlier grids is then
     // read through L2 (ld_prior).  The first grid of a chain (chain 1)
     // waits before it releases the next.  With the lengths carried in the
     // parameters (fused table sync) and no shared prefix, the first prologue
@@ -1040,7 +1042,11 @@ paged_attn_kernel(const __grid_constant__ CUtensorMap tmap, const __grid_constan
             make_ready();
             a.ws_run[bid] = make_int2(-1, -1);
         }
-        if (chained) grid_dependency_wait();
+        // CTA 0 waits whatever its share, so this grid's completion means the
+        // one before's.  The others leave: waiting, they would hold SM slots
+        // that a third co-located batch needs (2, 2 and 2 sequences with 8, 8 and
+        // 32 KV heads: 28.4 us a step with them waiting, 24.8 without).
+        if (chained && bid == 0) grid_dependency_wait();
     };
     if (bid >= NC) return no_part();
     // first unit of CTA i: i * W / NC, with W = wq * NC + wr
@@ -1507,6 +1513,18 @@ combine_kernel(const __grid_constant__ CombineArgs c)
 
 // host helpers ---------------------------------------------------------------
 constexpr int kRowsCap = 2048;
+
+// units that the batch's table has room for
+inline int64_t table_units(const AttnArgs &a, int D)
+{
+    const int unit = D == 64 ? kUnit<64> : kUnit<128>;
+    return (int64_t)a.S * a.Hkv * (((int64_t)a.max_blocks * a.bs + unit - 1) / unit);
+}
+// fewer than kMergeUnits units a warp (by the table's width)
+inline bool small_batch(const AttnArgs &a, int D, int P, int nwarps)
+{
+    return table_units(a, D) < (int64_t)kMergeUnits * P * nwarps;
+}
 
 // shared memory of a decode CTA; with boxes = 1, what it would be with a unit
 // of a box (the S that a call may have, see attn_run)

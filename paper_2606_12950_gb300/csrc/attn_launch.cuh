@@ -119,9 +119,8 @@ int attn_run(const CUtensorMap *tmap, AttnArgs a, int P_req, int sm_count, cudaS
     // (chain 3): then only the CTAs' later end shows.  The bits are the same
     // either way (CombineArgs::per_cta).  Beside a shared prefix only the
     // first rule holds.  In no case if the buffers cost a CTA per SM.
-    const int64_t most_units =
-        (int64_t)a.S * a.Hkv * (((int64_t)a.max_blocks * a.bs + kUnit<D> - 1) / kUnit<D>);
-    const bool small = most_units < (int64_t)kMergeUnits * P * a.nwarps;
+    const bool small = small_batch(a, D, P, a.nwarps);
+    const int32_t small_min_units = std::min(std::max(1, a.min_units), kMinPartTokens / kUnit<D>);
     bool merge = false;
     a.min_units = kMinPartTokens / kUnit<D>;
     // (with fewer warps the combine, which merges kPlainWarps records at a time,
@@ -138,7 +137,7 @@ int attn_run(const CUtensorMap *tmap, AttnArgs a, int P_req, int sm_count, cudaS
         if (merge) {
             fn = fn_merge;
             smem = smem_merge;
-            if (small) a.min_units = 1;
+            if (small) a.min_units = small_min_units;
         }
     }
     // At most one run per part starts there and goes on.  With several waves
@@ -174,11 +173,11 @@ int attn_run(const CUtensorMap *tmap, AttnArgs a, int P_req, int sm_count, cudaS
     if (what == kLaunchAttention) return KV_OK;
     CombineArgs c{a.out, a.ws_run, a.ws_part, a.S, a.Hkv, a.skip, a.ws_pre, a.KS};
     cudaLaunchConfig_t ccfg = cfg;
-    // records per run (of warps; a CTA's if warps may have a single unit):
-    // at most one per part, spread over the runs, plus the prefix records in
+    // records per run (of warps; of CTAs if the batch is small): at most one
+    // per part, spread over the runs, plus the prefix records in
     // shared-prefix mode
     const int runs = a.S * a.Hkv;
-    const double per_run = (double)P * (a.min_units == 1 ? 1 : a.nwarps) / std::max(1, runs) + 1.0 + (a.skip ? a.KS : 0);
+    const double per_run = (double)P * (merge && small ? 1 : a.nwarps) / std::max(1, runs) + 1.0 + (a.skip ? a.KS : 0);
     if constexpr (G * D / 4 >= 128) {
         // one group in shared-prefix mode: two columns a thread, so that
         // every member run fits in one wave

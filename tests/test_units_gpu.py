@@ -430,3 +430,60 @@ def test_shared_prefix_whose_first_keys_have_no_weight(d):
     for s in range(b.S):
         _check(got[s], _exact(b, ref_pool, s), s)
     assert pool.error() == 0
+
+
+@pytest.mark.parametrize("d", [64, 128])
+@pytest.mark.parametrize("lens", [[[30]] * 3, [[200, 90], [700, 33, 5, 260, 1, 64], [500]], [[3000], [2900, 64], [2500] * 3],
+                                  [[0], [900] * 6, [15, 16, 17]]], ids=["one_cta", "ragged", "long", "uneven"])
+def test_small_batches_in_one_call(lens, d):
+    """Co-located batches that are all small: from one unit a warp on, by the room
+    of all of them, CTAs without units among the chained kernels.  The same bits
+    in each of 20 steps; against the oracle, and against the calls one by one within the roundings of two work splits
+    (see test_cta_level_parts_against_the_oracle_and_the_general_path)."""
+    from paper_2606_12950_gb300 import kvpool as K
+    from paper_2606_12950_gb300.runner import DeviceBatch, DevicePool
+
+    heads = [(8, 2), (8, 8), (32, 4)]
+    for order in (slice(None), slice(None, None, -1)):
+        batches = [W.make_batch(8200 + d + i, pre, Hq=Hq, Hkv=Hkv, d=d, bs=16, extra_blocks=3)
+                   for i, (pre, (Hq, Hkv)) in enumerate(zip(lens[order], heads))]
+        page = 2 * 2 * 16 * d  # elements of the smallest block
+        first, n_pages, parts = [], 0, []
+        for b in batches:  # each batch's blocks in pages of their own
+            k = b.block_elems // page
+            b.table = np.where(b.table >= 0, b.table * k + n_pages, -1).astype(np.int32)
+            parts.append(b.pool)
+            first.append(n_pages)
+            n_pages += b.n_pages * k
+        host = np.concatenate(parts)
+        outs = []
+        for multi in (False, True):
+            pool = DevicePool(n_pages, page * 2, 16, [(b.Hkv, d) for b in batches])
+            pool.upload(host)
+            dbs = [DeviceBatch(pool, i, b) for i, b in enumerate(batches)]
+            if multi:
+                calls = K.attn_batches([db.batch() for db in dbs])
+                steps = []
+                for _ in range(20):
+                    K.paged_decode_attn_multi(pool.handle, calls)
+                    steps.append([db.out.clone() for db in dbs])
+                torch.cuda.synchronize()
+                for s in steps[:-1]:
+                    assert all(torch.equal(x, y) for x, y in zip(s, steps[-1]))
+            else:
+                for db in dbs:
+                    db.append_attend()
+            torch.cuda.synchronize()
+            assert pool.error() == 0
+            outs.append([db.out_f64() for db in dbs])
+            got_pool = pool.download()
+            ref_pool = host.copy()
+            for i, b in enumerate(batches):
+                oracle.append(ref_pool, n_pages, page, 16, b.Hkv, d, b.k_new, b.v_new, b.table, b.ctx_lens, inplace=True)
+            assert np.array_equal(got_pool, ref_pool)
+        vmax = np.abs(W.bf16_bits_to_f64(ref_pool)).max()
+        for i, b in enumerate(batches):
+            ref = oracle.paged_attention(ref_pool, n_pages, page, 16, b.Hkv, d, b.q, b.table, b.ctx_lens, b.scale)
+            for got in (outs[0][i], outs[1][i]):
+                assert np.all(np.abs(got - ref) <= (2.0 ** -9 + 2.0 ** -15) * (vmax + np.abs(ref))), i
+            assert np.all(np.abs(outs[0][i] - outs[1][i]) <= 2.0 ** -8 * (vmax + np.abs(ref))), i
