@@ -92,8 +92,10 @@ def _attend(b, max_blocks=None):
 def test_combine_with_few_and_many_runs(S, G, d):
     """One KV head, so S runs: either side of the lines at which the combine
     spreads a run's columns over 8, 4 or 1 CTAs (152 SMs), with runs of one
-    record and of several hundred."""
-    lens = [5000 if S < 3 else 700] + [17 + 41 * s % 333 for s in range(1, S)]
+    record and, with one or two sequences, of several hundred: 60000 tokens are
+    six units or more for each of 304 CTAs, more records than the 16 groups of
+    a combine CTA take at once (8 each)."""
+    lens = [60000 if S < 3 else 700] + [17 + 41 * s % 333 for s in range(1, S)]
     b = W.make_batch(7100 + S + G, lens, Hq=G, Hkv=1, d=d, bs=16, extra_blocks=3)
     pool, db = _attend(b)
     ref_pool = oracle.batch_append(b)
