@@ -473,9 +473,9 @@ int kv_append(kv_pool *pool, int layout, const uint16_t *k_new, const uint16_t *
 
 /*
  * Bytes of device workspace paged_decode_attn needs for these sizes and this
- * num_splits: one (first part, part count) pair of int32 per (sequence, KV
- * head) run, followed by fp32 split partials, one record of G*d + 2*G floats
- * per (run, part) pair a split run can produce.  Every call writes all it reads, so the
+ * num_splits: a run table, two int32 per (sequence, KV head) run that say
+ * where its records are, followed by fp32 split partials, one record of
+ * G*d + 2*G floats per (run, part) pair a split run can produce.  Every call writes all it reads, so the
  * workspace needs no initialisation and may be reused freely by calls that
  * are ordered on one stream.
  */
@@ -501,13 +501,15 @@ int kv_workspace_clear(void *workspace, size_t ws_bytes, void *stream);
  * are device memory.  A sequence with n == 0 gets zeros.
  * Arithmetic: fp32 products and accumulation, online softmax in base 2,
  * bf16 output rounded to nearest-even.
- * Work split: the batch's KV is cut into 16-token tiles of one (sequence,
- * KV head); the tiles are split into equal contiguous parts, one per warp of
- * the resident CTAs (num_splits == 0), or into num_splits * 8 parts when
- * num_splits > 0 CTAs are requested.  A (sequence, head) whose tiles fall in
- * more than one part leaves fp32 partials (max, sum, unnormalised output)
- * that a second kernel merges in part order, so results do not depend on
- * where blocks sit in the pool.  Launches two kernels on `stream`.
+ * Work split: the batch's KV is cut into tiles of one (sequence, KV head),
+ * 16 tokens at d = 128 and 32 at d = 64; the tiles are split into equal
+ * contiguous ranges, one per resident CTA (num_splits == 0) or per requested
+ * one (num_splits > 0), and a CTA's into equal ranges of its warps.  A
+ * (sequence, head) whose tiles fall in more than one part (a warp's range, or
+ * a CTA's, whose warps merge) leaves fp32 partials (max, sum, unnormalised
+ * output) that a second kernel merges in an order that only the lengths set,
+ * so results do not depend on where blocks sit in the pool.  A token whose
+ * score is -inf has no weight; one whose score is NaN makes the output NaN.  Launches two kernels on `stream`.
  * Errors: KV_ERR_INVALID_ARG, KV_ERR_UNSUPPORTED (d not 64/128, G not in
  * {1,2,4,5,8}, block size not a multiple of 16), KV_ERR_WORKSPACE.
  */

@@ -117,8 +117,8 @@ int attn_run(const CUtensorMap *tmap, AttnArgs a, int P_req, int sm_count, cudaS
     // the same bits whether the lengths come with it or not.  Larger batches
     // merge too, unless the next step's decode kernel overlaps the combine
     // (chain 3): then only the CTAs' later end shows.  The bits are the same
-    // either way (CombineArgs::per_cta).  Beside a shared prefix only the
-    // first rule holds.  In no case if the buffers cost a CTA per SM.
+    // either way (the combine merges a CTA's records first).  Beside a shared
+    // prefix only the first rule holds.  In no case if the buffers cost a CTA per SM.
     const bool small = small_batch(a, D, P, a.nwarps);
     const int32_t small_min_units = std::min(std::max(1, a.min_units), kMinPartTokens / kUnit<D>);
     bool merge = false;

@@ -364,8 +364,8 @@ int cascade_plan_run(const int32_t *words, int n_words, int S, int32_t *ws_plan,
     return cascade_plan_launch<kvp::kCascadeWords>(words, n_words, S, ws_plan, ws_skip, sync, ov, st);
 }
 
-// workspace: per-run (first part, parts) as int2 (padded to 256 bytes),
-// then the fp32 partials
+// workspace: the run table (AttnArgs::ws_run, an int2 per run, padded to 256
+// bytes), then the fp32 partials
 size_t ws_layout(int S, int Hkv, int G, int D, int P, size_t *part_off)
 {
     const size_t hdr = ((size_t)S * Hkv * sizeof(int2) + 255) / 256 * 256;
@@ -565,7 +565,7 @@ int attn_call(kv_pool *p, int layout, const uint16_t *q, const uint16_t *k_new, 
     // kernel's parameters, then launch, in stream order: the plan kernel
     // (per-sequence skips), the prefix kernel, the decode kernel over the
     // suffixes and the combine.  The prefix kernel takes about a quarter of
-    // the SMs (one CTA each); the decode kernel, sized to the SMs left, runs
+    // the SMs (one CTA each), up to 3/7 where it would end last; the decode kernel, sized to the SMs left, runs
     // beside it without waiting for it and waits for it at its end, so the
     // combine, which waits for the decode grid, sees both grids' records ----
     const int bs = p->desc.block_size, Hkv = L.num_kv_heads;
@@ -636,17 +636,25 @@ int attn_call(kv_pool *p, int layout, const uint16_t *q, const uint16_t *k_new, 
     // Key splits: as many as keep the prefix grid within a quarter of the
     // GPU's CTA slots for it (at least one; every split non-empty).  If a split
     // would still take longer than the suffixes beside it, more, up to 3/7 of
-    // the slots (64 SMs).  The lengths are on the device, so the suffixes are
-    // taken for kSuffixGuess tokens each.  A split takes about kSplitUs plus
+    // the slots (64 SMs).  The lengths are on the device (the sequence table's
+    // calls have them on the host too, but give the same bits as the others, so
+    // the same splits), and the suffixes are taken for kSuffixGuess tokens each.
+    // A split takes about kSplitUs plus
     // kKeyTileUs per 128 keys.  Measured, one step in us, at the quarter's
     // rule and at this one (splits): 190 suffixes of about 500 tokens, 3
     // groups, 4096-token prefixes 115 (1) and 84 (2); 200 of about 500, one
     // 8192-token prefix 192 (1) and 95 (2); 128 of about 100, 2 groups, 4096
     // tokens 57 (2) and 46 (3); 12 of about 500, 4096 tokens 30 (4) and 21 (8);
-    // 120 of about 2900, 3 groups, 4096 tokens 261 (1) and 259 (2).  Where the
-    // suffixes are much longer than the guess it can cost them a little: 361
-    // of about 3900, 4 groups, 3968 tokens, one KV head at d = 64, 69.7 (4)
-    // and 71.8 (8).  Past 3/7 the suffixes lose more than the prefix gains
+    // 120 of about 2900, 3 groups, 4096 tokens 261 (1) and 259 (2).  (Those with
+    // an earlier prefix kernel, 1.3 times as long a tile; with this one, 200 of
+    // about 500, one 8192-token prefix 146 (1) and 84 (2), 12 of about 500, 8192
+    // tokens 39 (4) and 27 (8).)  Where the suffixes are much longer than the
+    // guess it costs them something, at d = 64 more, as a tile takes less there
+    // than kKeyTileUs: one KV head, 361 of about 3900, 4 groups, 3968 tokens, 68.0
+    // (4) and 68.8 (8), and at d = 128 360 of about 3500 120.3 and 121.4; 8 query
+    // and 8 KV heads at d = 64, 360 of about 3500, 3 groups, 4096 tokens 556 (1)
+    // and 596 (2); and where the prefix is short: 12 of about 500, 1024 tokens
+    // 16.1 (4) and 16.9 (8).  Past 3/7 the suffixes lose more than the prefix gains
     // (8192 tokens: 113 with 4 splits on 128 SMs), and so they do where the
     // prefix is no longer than they are (256 of about 500 tokens, 2048-token
     // prefix: 101 with 1 split, 108 with 2).
