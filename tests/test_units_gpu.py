@@ -489,3 +489,32 @@ def test_small_batches_in_one_call(lens, d):
             for got in (outs[0][i], outs[1][i]):
                 assert np.all(np.abs(got - ref) <= (2.0 ** -9 + 2.0 ** -15) * (vmax + np.abs(ref))), i
             assert np.all(np.abs(outs[0][i] - outs[1][i]) <= 2.0 ** -8 * (vmax + np.abs(ref))), i
+
+
+@pytest.mark.parametrize("splits", [303, 305, 700, 3000])
+@pytest.mark.parametrize("lens", [[8000], [40, 700, 3, 1500, 64, 333, 900, 1999], [s % 40 for s in range(60)]],
+                         ids=["one", "some", "short"])
+@pytest.mark.parametrize("G,Hkv,d", [(4, 8, 128), (5, 2, 64)])
+def test_more_splits_than_resident_ctas(G, Hkv, d, lens, splits):
+    """num_splits either side of the CTAs that are resident (304 on 152 SMs) and far
+    above, in small batches: against the oracle (the bound of the roundings, see
+    above), and the same bits overlapping another call's combine."""
+    from paper_2606_12950_gb300.runner import DeviceBatch, DevicePool
+
+    b = W.make_batch(8300 + G, lens, Hq=G * Hkv, Hkv=Hkv, d=d, bs=16, extra_blocks=3)
+    pool = DevicePool(b.n_pages, b.page_elems * 2, b.bs, [(Hkv, d)])
+    pool.upload(b.pool)
+    db = DeviceBatch(pool, 0, b, splits)
+    db.append_attend()
+    torch.cuda.synchronize()
+    alone, ref_pool = db.out_bits(), oracle.batch_append(b)
+    assert np.array_equal(pool.download(), ref_pool)
+    ref = oracle.batch_attention(b, pool=ref_pool)
+    vmax = np.abs(W.bf16_bits_to_f64(ref_pool)).max()
+    assert np.all(np.abs(db.out_f64() - ref) <= (2.0 ** -9 + 2.0 ** -15) * (vmax + np.abs(ref)))
+    pool.set_step_overlap(True)
+    for _ in range(3):
+        db.append_attend()
+    torch.cuda.synchronize()
+    assert np.array_equal(alone, db.out_bits())
+    assert pool.error() == 0
