@@ -557,8 +557,8 @@ int paged_decode_attn_seqtab(kv_pool *pool, kv_seqtab *t, const uint16_t *q, con
  * layout, queries, tables and workspace, attending over the one pool.  The
  * result is that of calling paged_decode_attn (k_new / v_new NULL) or
  * paged_decode_attn_append for batches[0], batches[1], ... in order, with
- * num_splits = 0; where all the batches are small (their tables have room
- * for fewer than 8 units a warp), up to the rounding of another work split.
+ * num_splits = 0; for small batches (tables with room for fewer than 8 units
+ * a warp) beside each other, up to the rounding of another work split.
  * The decode kernels run as a chain: each later batch's kernel starts on the
  * SMs the one before frees as its last warps finish, and the split-K merges
  * of all batches follow.  Batches must not share a workspace or an output,

@@ -859,34 +859,36 @@ int paged_decode_attn_multi(kv_pool *p, int n, const kv_attn_batch *batches, voi
         return dispatch(it.variant, it.D, it.G, &p->tmap[it.layout], &it.a, it.P, p->sm_count, st,
                         kvp::kLaunchBoth, &P);
     }
-    // Batches that are all small run side by side if their CTAs fit on the GPU
-    // together, so a warp has at least as many units as shares the room of all
-    // among the GPU's warps (in attn_run, the part's least tokens at most).  With
-    // single units, as each batch has alone, the later kernels waited for the
-    // first one's CTAs: 2 and 5 sequences with 2 and 32 KV heads 18.5 us a step
-    // before small batches had them, 19.3 with them and 14.8 this way; 6 and 6
-    // of 700 tokens with 8 heads 19.0, 22.2 and 17.9; 1 and 8 with 32 and 2
-    // heads 20.5, 21.4 and 18.8; but 6 and 6 of very unequal lengths, for which
+    // Small batches run side by side if their CTAs fit on the GPU together, so a
+    // warp has at least as many units as shares the room of all of them among the
+    // GPU's warps (in attn_run, the part's least tokens at most).  With single
+    // units, as each batch has alone, the later kernels waited for the earlier
+    // one's CTAs: 2 and 5 sequences with 2 and 32 KV heads 18.5 us a step before
+    // small batches had them, 19.3 with them and 14.8 this way; 6 and 6 of 700
+    // tokens with 8 heads 19.0, 22.2 and 17.9; 1 and 8 with 32 and 2 heads 20.5,
+    // 21.4 and 18.8; two small ones of 6 and 8 beside a large one of 8 with 32
+    // heads 43.3, 44.0 and 39.5; but 6 and 6 of very unequal lengths, for which
     // the room says little, 19.4, 16.1 and 18.3.
     int64_t units = 0, warps = 1;
-    bool small = true;
+    size_t n_small = 0;
     for (const MultiItem &it : items) {
-        units += kvp::table_units(it.a, it.D);
         warps = std::max(warps, (int64_t)it.P * kvp::kPlainWarps);
-        small = small && kvp::small_batch(it.a, it.D, it.P, kvp::kPlainWarps);
+        if (!kvp::small_batch(it.a, it.D, it.P, kvp::kPlainWarps)) continue;
+        units += kvp::table_units(it.a, it.D);
+        ++n_small;
     }
-    if (small) {
-        for (MultiItem &it : items)
+    if (n_small > 1) {
+        for (MultiItem &it : items)  // (attn_run takes it for the small ones)
             it.a.min_units = (int32_t)std::min<int64_t>((units + warps - 1) / warps, kvp::kMinPartTokens);
     }
-    // Others the largest first, by the room in its table: a later kernel's CTAs
-    // start as the one before frees SMs, so its CTAs' starts and ends spread as
-    // much as those of all before it; a short one last leaves that spread short
-    // work.  Three co-located models (1.2, 0.3 and 0.1 GB): 267 us with the
-    // smallest first, 262 with the largest first; two of 30 and 110 MB 36.0 and
-    // 34.9.  Small ones stay in the caller's order: the smaller first is the
-    // better there, 17.3 and 18.8 for the 1 and 8 above.
-    if (!small)
+    // The largest first, by the room in its table: a later kernel's CTAs start
+    // as the one before frees SMs, so its CTAs' starts and ends spread as much
+    // as those of all before it; a short one last leaves that spread short work.
+    // Three co-located models (1.2, 0.3 and 0.1 GB): 267 us with the smallest
+    // first, 262 with the largest first; two of 30 and 110 MB 36.0 and 34.9.
+    // Where all are small they stay in the caller's order: the smaller first is
+    // the better there, 17.3 and 18.8 for the 1 and 8 above.
+    if (n_small < items.size())
         std::stable_sort(items.begin(), items.end(), [](const MultiItem &x, const MultiItem &y) {
             auto room = [](const MultiItem &i) { return (int64_t)i.a.S * i.a.Hkv * i.D * i.a.max_blocks; };
             return room(x) > room(y);

@@ -436,10 +436,11 @@ def test_shared_prefix_whose_first_keys_have_no_weight(d):
 
 @pytest.mark.parametrize("d", [64, 128])
 @pytest.mark.parametrize("lens", [[[30]] * 3, [[200, 90], [700, 33, 5, 260, 1, 64], [500]], [[3000], [2900, 64], [2500] * 3],
-                                  [[0], [900] * 6, [15, 16, 17]]], ids=["one_cta", "ragged", "long", "uneven"])
+                                  [[0], [900] * 6, [15, 16, 17]], [[100, 600], [30, 500, 7], [20] * 39 + [3900]]],
+                         ids=["one_cta", "ragged", "long", "uneven", "beside_a_large_one"])
 def test_small_batches_in_one_call(lens, d):
-    """Co-located batches that are all small: from one unit a warp on, by the room
-    of all of them, CTAs without units among the chained kernels.  The same bits
+    """Co-located batches that are small: from one unit a warp on, by the room of
+    all of them, CTAs without units among the chained kernels.  The same bits
     in each of 20 steps; against the oracle, and against the calls one by one within the roundings of two work splits
     (see test_cta_level_parts_against_the_oracle_and_the_general_path)."""
     from paper_2606_12950_gb300 import kvpool as K
