@@ -633,31 +633,30 @@ int attn_call(kv_pool *p, int layout, const uint16_t *q, const uint16_t *k_new, 
     int P_pre = 0;
     rc = cascade_dispatch(L.head_dim, G, nullptr, c, 0, p->sm_count, nullptr, false, &P_pre);
     if (rc) return rc;
-    // Key splits: as many as keep the prefix grid within a quarter of the
-    // GPU's CTA slots for it (at least one; every split non-empty).  If a split
-    // would still take longer than the suffixes beside it, more, up to 3/7 of
-    // the slots (64 SMs).  The lengths are on the device (the sequence table's
-    // calls have them on the host too, but give the same bits as the others, so
-    // the same splits), and the suffixes are taken for kSuffixGuess tokens each.
-    // A split takes about kSplitUs plus
-    // kKeyTileUs per 128 keys.  Measured, one step in us, at the quarter's
-    // rule and at this one (splits): 190 suffixes of about 500 tokens, 3
-    // groups, 4096-token prefixes 115 (1) and 84 (2); 200 of about 500, one
-    // 8192-token prefix 192 (1) and 95 (2); 128 of about 100, 2 groups, 4096
-    // tokens 57 (2) and 46 (3); 12 of about 500, 4096 tokens 30 (4) and 21 (8);
-    // 120 of about 2900, 3 groups, 4096 tokens 261 (1) and 259 (2).  (Those with
-    // an earlier prefix kernel, 1.3 times as long a tile; with this one, 200 of
-    // about 500, one 8192-token prefix 146 (1) and 84 (2), 12 of about 500, 8192
-    // tokens 39 (4) and 27 (8).)  Where the suffixes are much longer than the
-    // guess it costs them something, at d = 64 more, as a tile takes less there
-    // than kKeyTileUs: one KV head, 361 of about 3900, 4 groups, 3968 tokens, 68.0
-    // (4) and 68.8 (8), and at d = 128 360 of about 3500 120.3 and 121.4; 8 query
-    // and 8 KV heads at d = 64, 360 of about 3500, 3 groups, 4096 tokens 556 (1)
-    // and 596 (2); and where the prefix is short: 12 of about 500, 1024 tokens
-    // 16.1 (4) and 16.9 (8).  Past 3/7 the suffixes lose more than the prefix gains
-    // (8192 tokens: 113 with 4 splits on 128 SMs), and so they do where the
-    // prefix is no longer than they are (256 of about 500 tokens, 2048-token
-    // prefix: 101 with 1 split, 108 with 2).
+    // Key splits: as many as keep the prefix grid within a quarter of the GPU's
+    // CTA slots for it (at least one; every split non-empty).  If a split would
+    // still take longer than the suffixes beside it, more, up to 3/7 of the slots
+    // (64 SMs).  The lengths are on the device (the sequence table's calls have
+    // them on the host too, but give the same bits as the others, so the same
+    // splits), and the suffixes are taken for kSuffixGuess tokens each. A split
+    // takes about kSplitUs plus kKeyTileUs per 128 keys.  Measured, one step in
+    // us, at the quarter's rule and at this one (splits): 190 suffixes of about
+    // 500 tokens, 3 groups, 4096-token prefixes 115 (1) and 84 (2); 200 of about
+    // 500, one 8192-token prefix 192 (1) and 95 (2); 128 of about 100, 2 groups,
+    // 4096 tokens 57 (2) and 46 (3); 12 of about 500, 4096 tokens 30 (4) and 21
+    // (8); 120 of about 2900, 3 groups, 4096 tokens 261 (1) and 259 (2).  (Those
+    // with an earlier prefix kernel, 1.3 times as long a tile; with this one, 200
+    // of about 500, one 8192-token prefix 146 (1) and 84 (2), 12 of about 500,
+    // 8192 tokens 39 (4) and 27 (8).)  Where the suffixes are much longer than
+    // the guess it costs them something, at d = 64 more, as a tile takes less
+    // there than kKeyTileUs: one KV head, 361 of about 3900, 4 groups, 3968
+    // tokens, 68.0 (4) and 68.8 (8), and at d = 128 360 of about 3500 120.3 and
+    // 121.4; 8 query and 8 KV heads at d = 64, 360 of about 3500, 3 groups, 4096
+    // tokens 556 (1) and 596 (2); and where the prefix is short: 12 of about 500,
+    // 1024 tokens 16.1 (4) and 16.9 (8).  Past 3/7 the suffixes lose more than
+    // the prefix gains (8192 tokens: 113 with 4 splits on 128 SMs), and so they
+    // do where the prefix is no longer than they are (256 of about 500 tokens,
+    // 2048-token prefix: 101 with 1 split, 108 with 2).
     const int pre_base = std::max(1, tiles * Hkv);
     const int ks_most = std::min(kvp::kMaxKeySplits, kt_min);
     c->KS = std::max(1, std::min(P_pre / 4 / pre_base, ks_most));
